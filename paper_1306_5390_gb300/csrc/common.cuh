@@ -46,6 +46,10 @@ struct Ctrl {
     // counts every image pixel, a list pass the pixels it claimed), by kernel.
     unsigned long long evals_fused;
     unsigned long long evals_list;
+    // List-pass launch: pixels changed by the last pass it ran, and the state
+    // that the passes of one CTA alone leave to the others (k, list length).
+    int n_diff;
+    unsigned solo_k, solo_n;
 };
 
 // Grid barrier of the list-pass loop: two 64-bit counters on their own
@@ -129,12 +133,14 @@ struct PassArgs {
     // (xb, yb).  img_k[i], when set, receives image i's k: the number of the
     // last pass that changed one of its pixels (all images run the same
     // passes, and an image that a pass leaves unchanged is at a fixed point).
+    // img_n[i], set with it: image i's pixels changed by the last list pass.
     const ImgDesc* imgs;
     int nimg;
     int xb, yb;
     const int* tile_img;
     long long bm_total;       // words in one bitmap arena
     unsigned* img_k;
+    int* img_n = nullptr;
     int ntiles;               // fused-kernel tiles (all images)
     // Hybrid schedule: fused launch L (L = fused launches that ran before
     // it) writes change set L % 4, reads set (L + 3) % 4 and clears set

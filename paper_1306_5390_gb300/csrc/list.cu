@@ -1,29 +1,64 @@
 // List passes: passes of Algorithms 1-2 that evaluate only the pixels that
-// can change, all run by one persistent (cooperative) launch.
+// can differ from what their output canvas already holds, all run by one
+// persistent (cooperative) launch.
 //
-// A pixel's output in pass t depends only on its (2 beta + 1)^2 window in the
-// image of pass t-1, so a pixel with no changed pixel (in pass t-1) within
-// beta keeps its value.  Each pass walks the list of pixels the previous
-// pass changed and evaluates every pixel q within beta of one of them once,
-// by the changed pixel p that "owns" q: the first changed pixel, in raster
-// order, of q's window (read from the previous pass's change bitmap).  For
-// beta 1 one thread takes one changed pixel p, loads its 5 x 5
-// neighbourhood and evaluates the pixels of p's 3 x 3 window that p owns
-// from registers.  For wider windows one thread takes one (changed
+// Write I_t for the image after pass t.  Pass t + 1 reads I_t (canvas `cur`)
+// and turns canvas `aux`, which holds I_(t-1), into I_(t+1).  A pixel's value
+// in I_(t+1) depends only on its (2 beta + 1)^2 window in I_t, exactly as its
+// value in I_(t-1) depended on that window in I_(t-2).  So a pixel q must be
+// evaluated only if its window holds a pixel where I_t differs from I_(t-2);
+// everywhere else I_(t+1)(q) = I_(t-1)(q) is in place already.  The list a
+// pass reads is therefore D_t = {p : I_t(p) != I_(t-2)(p)}: the owner of q
+// compares its new value with the one it finds in `aux` and, if they differ,
+// writes it and appends q to D_(t+1).  Pixels that alternate between two
+// values (a large part of the impulses never settles in another way) leave
+// the lists, and the lists shrink by a factor of two to three per pass instead
+// of staying at the number of oscillating pixels (8192 x 8192, 30 %
+// impulses, beta 1: 24 passes evaluate 1.1 M pixels instead of 13.4 M, 0.164 ms
+// instead of 0.315; beta 2, 28 passes: 10.3 M instead of 21.4 M, 0.320 ms instead
+// of 0.520; 1920 x 1080, beta 2: 0.078 ms instead of 0.180).
+//
+// The first pass reads the fused launch's list C_t = {p : I_t(p) != I_(t-1)(p)}.
+// It serves as well (a pixel with no such p in its window keeps I_t(q) =
+// I_(t-1)(q)), and a pass that reads C_t finds every pixel of C_(t+1) and of
+// D_(t+1) and can make either; a pass that reads D_t can make only D_(t+1).  D_t
+// holds C_(t-1)'s settled pixels too, so while the changes still die out
+// quickly C is the shorter list.  A pass therefore makes C again while
+// the last list was shorter than 3/5 of the one before it (beta 5, 1000 x
+// 1500, 2 % impulses: 1.5 M evaluations against 2.8 M with D from the first
+// pass on); the first pass, which knows no ratio, makes D when the fused
+// launches ran kDirectD passes, by then the changes left are mostly
+// oscillations.
+//
+// k and the converged flag need to know whether a pass changed the image,
+// N_t = #{q : I_t(q) != I_(t-1)(q)} > 0.  For a pixel that is not evaluated
+// the inequality holds for pass t + 1 as it did for pass t, so N_(t+1) = N_t
+// + sum over the evaluated q of [I_(t+1)(q) != I_t(q)] - [I_t(q) !=
+// I_(t-1)(q)].  (A pass that reads C_t evaluates every changed pixel: the first
+// terms alone.)  When a D list comes out empty, the image alternates
+// between the two canvases for good: N = 0 means that the passes before this
+// one and its predecessor were the last to change anything, N > 0 that every
+// further pass changes the image, so k = max_k and the parity of the passes
+// left names the canvas.
+//
+// Every pixel q within beta of a listed pixel is evaluated once, by the listed
+// pixel p that "owns" q: the first one, in raster order, of q's window (read
+// from the list's bitmap).  For beta 1 one thread takes one listed pixel
+// p, loads its 5 x 5 neighbourhood and evaluates the pixels of p's 3 x 3 window
+// that p owns from registers.  For wider windows one thread takes one (listed
 // pixel, window row) pair, decides ownership for the whole row from one
 // bitmap word per window row, and queues the owned pixels in shared memory;
 // the CTA then evaluates its queue with all threads, so the evaluations run
-// without idle lanes.  Results go to the
-// partner canvas, which already agrees with the current image at every pixel
-// that is not evaluated (see Ctrl); pixels that change form the next list and
-// bitmap.  When the previous list overflowed its capacity, the pass evaluates
-// and writes every pixel instead.
+// without idle lanes.  When a list overflowed its capacity, the pass evaluates
+// every pixel instead.
 //
 // Passes are separated by a grid-wide barrier (all CTAs are co-resident, by
-// cooperative launch).  Every CTA tracks k, the converged flag and the
+// cooperative launch).  Every CTA tracks k, the list lengths and the
 // current canvas itself from values that are final at the barrier, so one
 // barrier per pass suffices; four list/bitmap sets rotate so that each set
-// is reset or cleared only while no CTA can still touch it.  Waits at the
+// is reset or cleared only while no CTA can still touch it.  Short lists are
+// left to CTA 0 alone (solo_passes), which needs no grid barrier between its
+// passes.  Waits at the
 // barrier are bounded: after one to two seconds the kernel records an error and
 // returns, and the call reports HGRMS_ETIMEOUT.
 #include "common.cuh"
@@ -42,7 +77,8 @@ constexpr int kListThreads = 512;
 // gpu-scope acquire (thread 0) and CTA barrier order each thread's later
 // loads after every write of the previous pass - the pattern of a grid-wide
 // synchronisation, after which ordinary loads observe the other CTAs' writes.
-// Nothing a pass reads is written during the same pass.
+// Nothing a pass reads through L1 is written during the same pass; the output
+// canvas, which a pass reads and writes, is read from L2 (__ldcg).
 
 // Bits [start, start + 32) of a bitmap row (outside [0, 32 * nwords): 0).
 __device__ __forceinline__ uint32_t row_bits(const uint32_t* __restrict__ row, int nwords, int start) {
@@ -213,7 +249,161 @@ __device__ __forceinline__ void mark_image(uint32_t* bits, bool ch, unsigned img
     if (ch && (int)(__ffs(peers & bal) - 1) == lane) atomicOr(bits + (img >> 5), 1u << (img & 31));
 }
 
+// The three bytes p[0..2] of the output canvas, from L2.
+__device__ __forceinline__ uint32_t load3_cg(const uint8_t* p) {
+    const uintptr_t a = reinterpret_cast<uintptr_t>(p);
+    const uint32_t* q = reinterpret_cast<const uint32_t*>(a & ~uintptr_t(3));
+    return __funnelshift_r(__ldcg(q), __ldcg(q + 1), (uint32_t)(a & 3u) * 8u);
+}
+
+// Warp-collective: img_n[img] += d for every lane with d != 0 (one atomic per
+// distinct image).
+__device__ __forceinline__ void add_image(int* img_n, int d, unsigned img, int lane) {
+    if (!__any_sync(0xffffffffu, d != 0)) return;
+    const unsigned peers = __match_any_sync(0xffffffffu, d != 0 ? img : 0xffffffffu);
+    const int sum = __reduce_add_sync(peers, d);
+    if (d != 0 && sum != 0 && __ffs(peers) - 1 == lane) atomicAdd(img_n + img, sum);
+}
+
+// Solo passes: a list of n pixels is left to CTA 0 when n P <= kSoloEvals
+// (P = (2 beta + 1)^2).  A pass of a handful of pixels is all latency: across
+// the grid 5.6 us with 152 CTAs and 6.4 us with 304, of which the barrier, the
+// append counter's round trip and the bitmap lookups are most; in one CTA,
+// with the lists and the claims in shared memory, 1.25 us for 30 pixels of
+// beta 2 and 5.4 us at the limit (beta 1, 205 pixels, four rounds of the
+// CTA's threads).
+constexpr unsigned kDirectD = 6;
+constexpr int kSoloEvals = 2048;
+constexpr int kSoloHash = 2 * kSoloEvals;        // claim table, at most half full
+constexpr int kSoloPasses = 1024;                // then the other CTAs' waits end
+constexpr unsigned kSoloClear = 1u << 16;        // largest list whose bitmap CTA 0 clears
+
 }  // namespace
+
+// State of the passes that every CTA follows (see the header).
+struct LoopState {
+    int t;              // passes run by the whole grid (set rotation)
+    unsigned k;         // number of the last pass run
+    unsigned cur, aux;  // canvases of I_t and I_(t-1)
+    unsigned n_cur;     // entries of the list the next pass reads
+    unsigned n_last;    // entries of the list before it (its bitmap is cleared by the next pass)
+    bool c_list;        // the next pass reads C_t (else D_t)
+};
+
+// Passes run by CTA 0 alone, from a list of st.n_cur <= kSoloEvals / P
+// pixels, until a list comes out empty, k reaches max_k, a list is longer
+// than that or kSoloPasses passes have run (the other CTAs wait meanwhile, and
+// their wait is bounded).  One thread takes one (listed pixel, window
+// position) pair and claims its pixel in a hash table.  Lists and claims
+// live in shared memory; the change sets are left as the grid's passes
+// expect them: the list of the next pass in the set that held the first one,
+// every other bitmap empty (st.t and the append counters stand still; another
+// CTA may not have read them yet).  st is updated (thread-uniform); s_n is two
+// counters; dn accumulates this thread's share of the change of N.
+template <int B, bool kBatch>
+__device__ __forceinline__ void solo_passes(const PassArgs& a, const ImgDesc& one, const int base, const int xb,
+                                            const int yb, const unsigned max_k, LoopState& st, uint32_t* lists,
+                                            uint32_t* hash, unsigned* s_n, unsigned& evals, int& dn) {
+    constexpr int W = 2 * B + 1, P = W * W, NW = (W + 3) / 4;
+    const int tid = threadIdx.x;
+    uint32_t* list = lists;
+    uint32_t* next = lists + kSoloEvals;
+    {
+        // The list, and clean bitmaps for all sets.
+        const int si = (st.t + base) & 3, sc = (st.t + base + 3) & 3;
+        auto clear = [&](uint32_t* bm, uint32_t e) {
+            unsigned img;
+            int y, x;
+            unpack_entry(e, xb, yb, img, y, x);
+            const ImgDesc d = kBatch ? load_desc(a.imgs, img) : one;
+            bm[d.bm_off + (long long)y * d.bm_words + (x >> 5)] = 0u;
+        };
+        for (unsigned i = tid; i < st.n_cur; i += kListThreads) {
+            const uint32_t e = __ldcg(a.lists[si] + i);
+            list[i] = e;
+            clear(a.bitmaps[si], e);
+        }
+        for (unsigned i = tid; i < st.n_last; i += kListThreads) clear(a.bitmaps[sc], __ldcg(a.lists[sc] + i));
+    }
+    unsigned n = st.n_cur;
+    for (int passes = 1;; ++passes) {
+        for (int i = tid; i < kSoloHash; i += kListThreads) hash[i] = 0xffffffffu;
+        unsigned* nn = s_n + (passes & 1);  // the other one may still be read
+        if (tid == 0) *nn = 0u;
+        __syncthreads();
+        const uint8_t* in_arena = a.canvas[st.cur];
+        uint8_t* out_arena = a.canvas[st.aux];
+        const int ntask = (int)n * P;
+        for (int i = tid; i < ntask; i += kListThreads) {
+            const int e = i / P, o = i - e * P;
+            unsigned img;
+            int y, x;
+            unpack_entry(list[e], xb, yb, img, y, x);
+            const ImgDesc d = kBatch ? load_desc(a.imgs, img) : one;
+            y += o / W - B;
+            x += o % W - B;
+            if (y < B || y >= d.rows - B || x < B || x >= d.cols - B) continue;
+            // Claim q (an interior pixel never packs to the empty key: its row
+            // and column are not the last ones of the fields' ranges).
+            const uint32_t key = pack_entry(img, y, x, xb, yb);
+            unsigned slot = (key * 0x9E3779B1u) >> 16 & (kSoloHash - 1);
+            bool mine = false;
+            for (int probe = 0; probe < kSoloHash; ++probe) {
+                const uint32_t was = atomicCAS(&hash[slot], 0xffffffffu, key);
+                mine = was == 0xffffffffu;
+                if (mine || was == key) break;
+                slot = (slot + 1) & (kSoloHash - 1);
+            }
+            if (!mine) continue;
+            const long long off = d.off + (long long)(kPadY + y) * d.pitch + kPadX + x;
+            const uint8_t* in = in_arena + off;
+            const int was = __ldcg(out_arena + off);
+            uint32_t win[W][NW];
+#pragma unroll
+            for (int r = 0; r < W; ++r) load_row_bytes<W>(in + (long long)(r - B) * d.pitch - B, win[r]);
+            ++evals;
+            const int ip = (int)((win[B][B / 4] >> (8 * (B % 4))) & 0xffu);
+            const int nv = eval_window<B>(win, a.alpha);
+            if (nv != was) {
+                out_arena[off] = (uint8_t)nv;
+                next[atomicAdd(nn, 1u)] = key;
+            }
+            const int now = nv != ip ? 1 : 0, before = ip != was ? 1 : 0;
+            const int delta = now - (st.c_list ? 0 : before);
+            dn += delta;
+            if (kBatch && a.img_k) {
+                if (delta) atomicAdd(a.img_n + img, delta);
+                if (now || before) atomicMax(a.img_k + img, st.k + (unsigned)now);
+            }
+        }
+        __syncthreads();
+        n = *nn;
+        ++st.k;
+        st.c_list = false;
+        const unsigned c = st.cur;
+        st.cur = st.aux;
+        st.aux = c;
+        uint32_t* l = list;
+        list = next;
+        next = l;
+        if (n == 0u || st.k >= max_k || n * P > kSoloEvals || passes >= kSoloPasses) break;
+    }
+    st.n_cur = n;
+    st.n_last = 0u;
+    if (n != 0u && st.k < max_k) {
+        // The grid goes on from this list.
+        const int si = (st.t + base) & 3;
+        for (unsigned i = tid; i < n; i += kListThreads) {
+            const uint32_t e = list[i];
+            if (i < a.list_cap) a.lists[si][i] = e;
+            unsigned img;
+            int y, x;
+            unpack_entry(e, xb, yb, img, y, x);
+            const ImgDesc d = kBatch ? load_desc(a.imgs, img) : one;
+            atomicOr(a.bitmaps[si] + d.bm_off + (long long)y * d.bm_words + (x >> 5), 1u << (x & 31));
+        }
+    }
+}
 
 // kBatch = false: one image, described by the launch arguments (pitch, rows,
 // cols, bm_words; entries packed 16/16); true: the image table.
@@ -222,13 +412,19 @@ __global__ void __launch_bounds__(kListThreads, 2) list_loop_kernel(PassArgs a) 
     constexpr int W = 2 * B + 1, P = W * W;
     constexpr int kWarps = kListThreads / 32;
     __shared__ int s_np;
-    __shared__ unsigned s_k, s_cur, s_aux, s_maxk, s_gen, s_base;
-    __shared__ unsigned s_n, s_nclr, s_app;
-    __shared__ uint32_t stage_all[kWarps][StagedList::kCap];
+    __shared__ unsigned s_k, s_cur, s_aux, s_maxk, s_base;
+    __shared__ unsigned s_n, s_nclr, s_app, s_solo_n[2];
+    __shared__ int s_dn;
+    // Staged list entries, one buffer per warp; solo passes keep their two lists here.
+    __shared__ uint32_t stage_all[kWarps * StagedList::kCap];
+    static_assert(kWarps * StagedList::kCap >= 2 * kSoloEvals, "the solo lists fit the staging buffers");
     __shared__ int s_counts[kWarps + 1];
     __shared__ unsigned long long s_evals;
-    __shared__ uint32_t s_imgbits[kBatch ? kMaxBatchImages / 32 : 1];  // images changed in this pass (by this CTA)
-    __shared__ uint32_t s_queue[B == 1 ? 1 : kListThreads * W];  // pixels this CTA evaluates in the current chunk
+    // Images changed by this pass, and by the pass before it (both as this CTA saw).
+    __shared__ uint32_t s_imgbits[kBatch ? kMaxBatchImages / 32 : 1], s_imgbits0[kBatch ? kMaxBatchImages / 32 : 1];
+    // Pixels this CTA evaluates in the current chunk (beta >= 2); the claim table of the solo passes.
+    constexpr int kQueue = B == 1 ? 1 : kListThreads * W;
+    __shared__ uint32_t s_queue[kQueue > kSoloHash ? kQueue : kSoloHash];
     __shared__ int s_qn[2];  // queue lengths; chunks alternate between them
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     Ctrl* ctrl = a.ctrl;
@@ -241,20 +437,26 @@ __global__ void __launch_bounds__(kListThreads, 2) list_loop_kernel(PassArgs a) 
         s_cur = __ldcg(&ctrl->cur);
         s_aux = __ldcg(&ctrl->aux);
         s_maxk = __ldcg(&ctrl->max_k);
-        s_gen = 0u;  // barriers completed; the barrier struct is zeroed at the start of every call
         // The last fused launch wrote change set (fused launches - 1) % 4.
         s_base = (__ldcg(&ctrl->fused_work) + 3u) & 3u;
     }
     if constexpr (kBatch)
-        for (int i = tid; i < kMaxBatchImages / 32; i += kListThreads) s_imgbits[i] = 0u;
+        for (int i = tid; i < kMaxBatchImages / 32; i += kListThreads) s_imgbits[i] = s_imgbits0[i] = 0u;
     __syncthreads();
     if (s_np == 0) return;  // the fused launch already finished the call
-    unsigned k = s_k, cur = s_cur, aux = s_aux, gen = s_gen;
+    LoopState st;
+    st.t = 0;
+    st.k = s_k;
+    st.cur = s_cur;
+    st.aux = s_aux;
+    st.c_list = true;
+    unsigned n_before = 0;  // entries of the list that the previous pass read
+    unsigned gen = 0u;                // barriers completed; the barrier struct is zeroed at the start of every call
     unsigned prev_hi[2] = {0u, 0u};  // thread 0: counts seen at the last use of each barrier counter
     const int base = (int)s_base;
-    const unsigned max_k = s_maxk;
-    bool converged = false, failed = false;
-    int passes = 0;
+    const unsigned max_k = s_maxk, k0 = s_k;
+    const unsigned max_spins = a.bar_spins ? a.bar_spins : (1u << 22);
+    bool failed = false;
     unsigned evals = 0;
     int qpar = 0;  // queue counter of the next chunk (CTA-uniform)
     const long long gthreads = (long long)gridDim.x * blockDim.x;
@@ -275,36 +477,82 @@ __global__ void __launch_bounds__(kListThreads, 2) list_loop_kernel(PassArgs a) 
     }
     constexpr int kXb = 16, kYb = 16;
     const int xb = kBatch ? a.xb : kXb, yb = kBatch ? a.yb : kYb;
-    StagedList sl{stage_all[warp], 0, 0u};
-    // List lengths: n_cur = entries of the list this pass reads (appended by
-    // the previous pass), n_last = those of the list the previous pass read
-    // (whose bitmap this pass clears); later lengths come from the barrier.
+    StagedList sl{stage_all + warp * StagedList::kCap, 0, 0u};
+    // List lengths at the start; later ones come from the barrier.
     if (tid == 0) {
         s_n = __ldcg(&ctrl->list_n[base]);
         s_nclr = __ldcg(&ctrl->list_n[(base + 3) & 3]);
         s_app = 0u;
+        s_dn = 0;
     }
     __syncthreads();
-    unsigned n_cur = s_n, n_last = s_nclr;
+    st.n_cur = s_n;
+    st.n_last = s_nclr;
 
-    for (int t = 0; k < max_k; ++t) {
-        const int si = (t + base) & 3, so = (t + base + 1) & 3, sc = (t + base + 3) & 3;
-        const uint8_t* in_arena = a.canvas[cur];
-        uint8_t* out_arena = a.canvas[aux];
+    while (true) {
+        int dn = 0;  // this thread's share of the change of N
+        if (st.n_cur <= (unsigned)(kSoloEvals / P) && st.n_cur <= a.list_cap && st.n_last <= kSoloClear &&
+            st.n_last <= a.list_cap) {
+            if (blockIdx.x == 0) {
+                solo_passes<B, kBatch>(a, one, base, xb, yb, max_k, st, stage_all, s_queue, s_solo_n, evals, dn);
+                dn = __reduce_add_sync(0xffffffffu, dn);
+                if (lane == 0 && dn) atomicAdd(&s_dn, dn);
+                __syncthreads();
+                if (tid == 0) {
+                    s_qn[0] = s_qn[1] = 0;
+                    if (s_dn) atomicAdd(&ctrl->n_diff, s_dn);
+                    s_dn = 0;
+                    ctrl->solo_k = st.k;
+                    ctrl->solo_n = st.n_cur;
+                }
+            }
+            unsigned zero = 0;
+            if (!grid_barrier(a.bar, ctrl, gridDim.x, gen, &s_app, prev_hi, zero, a.bar_extra, max_spins)) {
+                failed = true;
+                break;
+            }
+            if (blockIdx.x != 0) {
+                if (tid == 0) {
+                    s_k = __ldcg(&ctrl->solo_k);
+                    s_n = __ldcg(&ctrl->solo_n);
+                }
+                __syncthreads();
+                const unsigned ran = s_k - st.k;
+                st.k = s_k;
+                st.n_cur = s_n;
+                st.n_last = 0u;
+                st.c_list = false;
+                if (ran & 1u) {
+                    const unsigned c = st.cur;
+                    st.cur = st.aux;
+                    st.aux = c;
+                }
+            }
+            if (st.n_cur == 0u || st.k >= max_k) break;
+            continue;
+        }
+        const int si = (st.t + base) & 3, so = (st.t + base + 1) & 3, sc = (st.t + base + 3) & 3;
+        const uint8_t* in_arena = a.canvas[st.cur];
+        uint8_t* out_arena = a.canvas[st.aux];
         const uint32_t* prev = a.lists[si];
         const uint32_t* bm_prev = a.bitmaps[si];
         uint32_t* next = a.lists[so];
         uint32_t* bm_next = a.bitmaps[so];
         unsigned* nnext = &ctrl->list_n[so];
+        // Which list this pass makes (see the header).
+        const bool make_c = st.c_list && (n_before == 0u ? k0 < kDirectD : (unsigned long long)st.n_cur * 5u < (unsigned long long)n_before * 3u);
+        // N is needed from the first D_t on: the pass that makes it counts the
+        // pixels it changes, the later ones the differences.
+        const int add = make_c ? 0 : 1, sub = st.c_list ? 0 : 1;
         if (tid == 0 && blockIdx.x == 0) {
             // Set (t + base + 2) % 4 is next written by pass t + 1; its list
             // was last read (to clear its bitmap) in pass t - 1.
-            ctrl->list_n[(t + base + 2) & 3] = 0u;
+            ctrl->list_n[(st.t + base + 2) & 3] = 0u;
         }
-        const unsigned n = n_cur, nclr = n_last;
-        // The first list entry this thread reads (beta 1: pair warp_base +
-        // lane; wider windows: task tid * gridDim.x + blockIdx.x), loaded
-        // before the bitmap clearing below so that the two loads overlap.
+        const unsigned n = st.n_cur, nclr = st.n_last;
+        // The first list entry this thread reads (beta 1: entry tid *
+        // gridDim.x + blockIdx.x; wider windows: the entry of that task),
+        // loaded before the bitmap clearing below so that the two loads overlap.
         uint32_t pk_first = 0u;
         if (n <= a.list_cap) {
             const long long i0 = (long long)tid * gridDim.x + blockIdx.x;
@@ -329,18 +577,20 @@ __global__ void __launch_bounds__(kListThreads, 2) list_loop_kernel(PassArgs a) 
             }
         }
         if (n <= a.list_cap && B == 1) {
-            // beta 1: one thread per changed pixel p.  It loads p's 5 x 5
-            // neighbourhood and the previous pass's change bits of the rows
-            // up to p's, and evaluates every pixel q of p's 3 x 3 window
-            // that p owns (no changed pixel of q's window precedes p in
-            // raster order) from those registers.  Changed pixels are dealt
-            // to the CTAs in turn.
+            // beta 1: one thread per listed pixel p.  It loads p's 5 x 5
+            // neighbourhood, the 3 x 3 window of the output canvas and the
+            // list's bits of the rows up to p's, and evaluates every pixel q
+            // of p's 3 x 3 window that p owns (no listed pixel of q's window
+            // precedes p in raster order) from those registers.  Listed
+            // pixels are dealt to the CTAs in turn.
             long long i = (long long)tid * gridDim.x + blockIdx.x;
             uint32_t pk = pk_first;
             for (long long c0 = 0; c0 + blockIdx.x < (long long)n; c0 += gthreads, i += gthreads) {
                 const long long inext = i + gthreads;
                 const uint32_t pk_next = inext < (long long)n ? __ldcg(prev + (unsigned)inext) : 0u;
-                uint32_t chm = 0u;  // bit (dy + 1) * 3 + dx + 1: q = p + (dy, dx) changed
+                uint32_t chm = 0u;  // bit (dy + 1) * 3 + dx + 1: q = p + (dy, dx) goes on the next list
+                int delta = 0;      // the change of N
+                bool now = false, before = false;
                 unsigned img = 0;
                 int py = 0, px = 0;
                 if (i < (long long)n) {
@@ -349,7 +599,7 @@ __global__ void __launch_bounds__(kListThreads, 2) list_loop_kernel(PassArgs a) 
                     const uint32_t* bmp = bm_prev + d.bm_off;
                     const uint8_t* in = in_arena + d.off + (long long)kPadY * d.pitch + kPadX;
                     uint8_t* out = out_arena + d.off + (long long)kPadY * d.pitch + kPadX;
-                    // Change bits of rows py - 2 .. py, columns px - 2 .. (bit j: column px - 2 + j).
+                    // List bits of rows py - 2 .. py, columns px - 2 .. (bit j: column px - 2 + j).
                     uint32_t rb[3];
 #pragma unroll
                     for (int r = 0; r < 3; ++r) {
@@ -357,18 +607,20 @@ __global__ void __launch_bounds__(kListThreads, 2) list_loop_kernel(PassArgs a) 
                         rb[r] = gy >= 0 ? row_bits(bmp + (size_t)gy * d.bm_words, d.bm_words, px - 2) : 0u;
                     }
                     // Rows py - 2 .. py + 2, bytes px - 2 .. px + 2 (the canvas padding keeps them in bounds).
-                    uint32_t nb[5][2];
+                    uint32_t nb[5][2], ob[3];
                     const long long off = (long long)py * d.pitch + px;
 #pragma unroll
                     for (int r = 0; r < 5; ++r) load_row_bytes<5>(in + off + (long long)(r - 2) * d.pitch - 2, nb[r]);
+#pragma unroll
+                    for (int r = 0; r < 3; ++r) ob[r] = load3_cg(out + off + (long long)(r - 1) * d.pitch - 1);
 #pragma unroll
                     for (int dy = -1; dy <= 1; ++dy)
 #pragma unroll
                         for (int dx = -1; dx <= 1; ++dx) {
                             const int qy = py + dy, qx = px + dx;
                             if (qy < 1 || qy >= d.rows - 1 || qx < 1 || qx >= d.cols - 1) continue;
-                            // Ownership: q's window rows above p's hold no change, and
-                            // p's row none left of p (bits dx + 1 .. 1).
+                            // Ownership: q's window rows above p's hold no listed pixel,
+                            // and p's row none left of p (bits dx + 1 .. 1).
                             bool owner = true;
 #pragma unroll
                             for (int r = dy + 1; r <= dy + 3; ++r) {
@@ -381,24 +633,35 @@ __global__ void __launch_bounds__(kListThreads, 2) list_loop_kernel(PassArgs a) 
                             for (int r = 0; r < 3; ++r)
                                 w3[r][0] = __funnelshift_r(nb[dy + 1 + r][0], nb[dy + 1 + r][1], 8 * (dx + 1));
                             const int ip = (int)((w3[1][0] >> 8) & 0xffu);
+                            const int was = (int)((ob[dy + 1] >> (8 * (dx + 1))) & 0xffu);
                             const int nv = eval_window<1>(w3, a.alpha);
                             ++evals;
-                            out[(long long)qy * d.pitch + qx] = (uint8_t)nv;
-                            if (nv != ip) {
+                            if (nv != was) out[(long long)qy * d.pitch + qx] = (uint8_t)nv;
+                            if (nv != (make_c ? ip : was)) {
                                 chm |= 1u << ((dy + 1) * 3 + dx + 1);
                                 atomicOr(bm_next + d.bm_off + (size_t)qy * d.bm_words + (qx >> 5), 1u << (qx & 31));
                             }
+                            delta += (nv != ip ? add : 0) - (ip != was ? sub : 0);
+                            if (kBatch) {
+                                now = now || nv != ip;
+                                before = before || ip != was;
+                            }
                         }
                 }
-                if (kBatch && a.img_k) mark_image(s_imgbits, chm != 0u, img, lane);
-                // Append the changed pixels (one warp scan per round).
+                dn += delta;
+                if (kBatch && a.img_k) {
+                    mark_image(s_imgbits, now, img, lane);
+                    mark_image(s_imgbits0, before && !now, img, lane);
+                    add_image(a.img_n, delta, img, lane);
+                }
+                // Append the pixels (one warp scan per round).
                 staged_append_mask(sl, next, nnext, a.list_cap, chm, lane, [&](int bt) {
                     return pack_entry(img, py + bt / 3 - 1, px + bt % 3 - 1, xb, yb);
                 });
                 pk = pk_next;
             }
         } else if (n <= a.list_cap) {
-            // Chunks of one task per thread: task (changed pixel p, window
+            // Chunks of one task per thread: task (listed pixel p, window
             // row dy) finds the pixels q = p + (dy, dx) that p owns and
             // queues them in shared memory (phase A); the CTA then evaluates
             // its queue with every thread (phase B).  Tasks are dealt to the
@@ -411,8 +674,8 @@ __global__ void __launch_bounds__(kListThreads, 2) list_loop_kernel(PassArgs a) 
             for (long long c0 = 0; c0 + blockIdx.x < ntask; c0 += gthreads, i += gthreads) {
                 const long long inext = i + gthreads;
                 const uint32_t pk_next = inext < ntask ? __ldcg(prev + (unsigned)(inext / W)) : 0u;
-                // Phase A.  Ownership: no changed pixel of q's window precedes
-                // p in raster order.  rb[r] = the previous pass's changes in
+                // Phase A.  Ownership: no listed pixel of q's window precedes
+                // p in raster order.  rb[r] = the list's bits in
                 // row qy - B + r, columns px - 2B .. px + 2B (bit j: column
                 // px - 2B + j); q = (qy, px + dx) has window columns bits
                 // dx + B .. dx + 3B, its rows above py must have none and row
@@ -433,18 +696,18 @@ __global__ void __launch_bounds__(kListThreads, 2) list_loop_kernel(PassArgs a) 
                             const int gy = qy - B + r;
                             rb[r] = (gy <= py) ? row_bits(bmp + (size_t)gy * d.bm_words, d.bm_words, px - 2 * B) : 0u;
                         }
-                        uint32_t before = 0u;
+                        uint32_t ahead = 0u;
 #pragma unroll
                         for (int r = 0; r <= 2 * B; ++r) {
                             const int gy = qy - B + r;
-                            if (gy < py) before |= rb[r];
-                            if (gy == py) before |= rb[r] & ((1u << (2 * B)) - 1u);
+                            if (gy < py) ahead |= rb[r];
+                            if (gy == py) ahead |= rb[r] & ((1u << (2 * B)) - 1u);
                         }
 #pragma unroll
                         for (int dx = -B; dx <= B; ++dx) {
                             const int qx = px + dx;
                             const uint32_t wm = ((1u << W) - 1u) << (dx + B);
-                            if (qx >= B && qx < d.cols - B && (before & wm) == 0u) own |= 1u << (dx + B);
+                            if (qx >= B && qx < d.cols - B && (ahead & wm) == 0u) own |= 1u << (dx + B);
                         }
                     }
                 }
@@ -475,30 +738,40 @@ __global__ void __launch_bounds__(kListThreads, 2) list_loop_kernel(PassArgs a) 
                 if (tid == 0) s_qn[qpar ^ 1] = 0;
                 for (int j0 = warp * 32; j0 < qn; j0 += kListThreads) {
                     const int j = j0 + lane;
-                    bool ch = false;
+                    bool ch = false, now = false, before = false;
                     uint32_t v = 0;
                     unsigned qimg = 0;
                     if (j < qn) {
                         int y, x;
-                        unpack_entry(s_queue[j], xb, yb, qimg, y, x);
+                        v = s_queue[j];
+                        unpack_entry(v, xb, yb, qimg, y, x);
                         const ImgDesc d = kBatch ? load_desc(a.imgs, qimg) : one;
                         const uint8_t* in = in_arena + d.off + (long long)kPadY * d.pitch + kPadX;
                         constexpr int NW = (W + 3) / 4;
                         uint32_t win[W][NW];
                         const long long off = (long long)y * d.pitch + x;
+                        uint8_t* out = out_arena + d.off + (long long)kPadY * d.pitch + kPadX + off;
+                        const int was = __ldcg(out);
 #pragma unroll
                         for (int r = 0; r < W; ++r) load_row_bytes<W>(in + off + (long long)(r - B) * d.pitch - B, win[r]);
                         ++evals;
                         const int ip = (int)((win[B][B / 4] >> (8 * (B % 4))) & 0xffu);
                         const int nv = eval_window<B>(win, a.alpha);
-                        out_arena[d.off + (long long)kPadY * d.pitch + kPadX + off] = (uint8_t)nv;
-                        if (nv != ip) {
+                        if (nv != was) *out = (uint8_t)nv;
+                        if (nv != (make_c ? ip : was)) {
                             ch = true;
-                            v = pack_entry(qimg, y, x, xb, yb);
                             atomicOr(bm_next + d.bm_off + (size_t)y * d.bm_words + (x >> 5), 1u << (x & 31));
                         }
+                        now = nv != ip;
+                        before = ip != was;
                     }
-                    if (kBatch && a.img_k) mark_image(s_imgbits, ch, qimg, lane);
+                    const int delta = (now ? add : 0) - (before ? sub : 0);
+                    dn += delta;
+                    if (kBatch && a.img_k) {
+                        mark_image(s_imgbits, now, qimg, lane);
+                        mark_image(s_imgbits0, before && !now, qimg, lane);
+                        add_image(a.img_n, delta, qimg, lane);
+                    }
                     staged_append(sl, next, nnext, a.list_cap, ch, v, lane);
                 }
                 __syncthreads();  // every thread has read the queue
@@ -506,88 +779,114 @@ __global__ void __launch_bounds__(kListThreads, 2) list_loop_kernel(PassArgs a) 
                 pk = pk_next;
             }
         } else {
-            // Previous list overflowed: evaluate and write every pixel of
-            // every image.
+            // The list overflowed: evaluate every pixel of every image.
             for (int im = 0; im < (kBatch ? a.nimg : 1); ++im) {
                 const ImgDesc d = kBatch ? load_desc(a.imgs, (unsigned)im) : one;
                 const uint8_t* in = in_arena + d.off + (long long)kPadY * d.pitch + kPadX;
                 uint8_t* out = out_arena + d.off + (long long)kPadY * d.pitch + kPadX;
                 const long long total = (long long)d.rows * d.cols;
-                for (long long base = warp_base; base < total; base += gthreads) {
-                    const long long i = base + lane;
-                    bool ch = false;
+                for (long long p0 = warp_base; p0 < total; p0 += gthreads) {
+                    const long long i = p0 + lane;
+                    bool ch = false, now = false, before = false;
                     uint32_t v = 0;
                     if (i < total) {
                         const int y = (int)(i / d.cols), x = (int)(i - (long long)y * d.cols);
                         const long long off = (long long)y * d.pitch + x;
                         ++evals;
-                        const int ip = in[off];
+                        const int ip = in[off], was = __ldcg(out + off);
                         int nv = ip;
                         if (y >= B && y < d.rows - B && x >= B && x < d.cols - B)
                             nv = eval_pixel<B>(in + off, d.pitch, a.alpha);
-                        out[off] = (uint8_t)nv;
-                        if (nv != ip) {
+                        if (nv != was) out[off] = (uint8_t)nv;
+                        if (nv != (make_c ? ip : was)) {
                             ch = true;
                             v = pack_entry((unsigned)im, y, x, xb, yb);
                             atomicOr(bm_next + d.bm_off + (size_t)y * d.bm_words + (x >> 5), 1u << (x & 31));
                         }
+                        now = nv != ip;
+                        before = ip != was;
                     }
-                        if (kBatch && a.img_k) mark_image(s_imgbits, ch, (unsigned)im, lane);
+                    const int delta = (now ? add : 0) - (before ? sub : 0);
+                    dn += delta;
+                    if (kBatch && a.img_k) {
+                        mark_image(s_imgbits, now, (unsigned)im, lane);
+                        mark_image(s_imgbits0, before && !now, (unsigned)im, lane);
+                        add_image(a.img_n, delta, (unsigned)im, lane);
+                    }
                     staged_append(sl, next, nnext, a.list_cap, ch, v, lane);
                 }
             }
         }
+        dn = __reduce_add_sync(0xffffffffu, dn);
+        if (lane == 0 && dn) atomicAdd(&s_dn, dn);
         staged_flush(sl, next, nnext, a.list_cap, s_counts, kWarps);
-        // Images this CTA changed in pass number k + 1 (staged_flush ends
-        // with a block barrier, so every mark is in place).
+        // Images this CTA saw changed by this pass (number k + 1) or the one
+        // before it (staged_flush ends with a block barrier, so every mark is
+        // in place).
         if (kBatch && a.img_k) {
             for (int w = tid; w < (a.nimg + 31) / 32; w += kListThreads) {
-                uint32_t bits = s_imgbits[w];
-                s_imgbits[w] = 0u;
+                const uint32_t now = s_imgbits[w];
+                uint32_t bits = now | s_imgbits0[w];
+                s_imgbits[w] = s_imgbits0[w] = 0u;
                 while (bits) {
                     const int b = __ffs(bits) - 1;
                     bits &= bits - 1u;
-                    a.img_k[32 * w + b] = k + 1u;
+                    atomicMax(a.img_k + 32 * w + b, st.k + ((now >> b) & 1u));
                 }
             }
         }
-        ++passes;
-        // Entries this CTA appended (every changed pixel appends one).
+        // Entries this CTA appended, and its share of the change of N.
         if (lane == 0 && sl.total) atomicAdd(&s_app, sl.total);
         sl.total = 0u;
+        if (tid == 0) {
+            if (s_dn) atomicAdd(&ctrl->n_diff, s_dn);  // s_dn is complete: staged_flush has block barriers
+            s_dn = 0;
+        }
         unsigned appended = 0;
-        if (!grid_barrier(a.bar, ctrl, gridDim.x, gen, &s_app, prev_hi, appended, a.bar_extra,
-                          a.bar_spins ? a.bar_spins : (1u << 22))) {
+        if (!grid_barrier(a.bar, ctrl, gridDim.x, gen, &s_app, prev_hi, appended, a.bar_extra, max_spins)) {
             failed = true;
             break;
         }
         if (tid == 0) s_app = 0u;  // read by thread 0 inside the barrier only
-        n_last = n_cur;
-        n_cur = appended;
-        if (appended == 0u) {
-            converged = true;  // a fixed point: the output canvas equals the input
-            break;
-        }
-        ++k;
-        const unsigned tmp = cur;
-        cur = aux;
-        aux = tmp;
+        ++st.t;
+        ++st.k;
+        st.c_list = make_c;
+        n_before = st.n_cur;
+        const unsigned c = st.cur;
+        st.cur = st.aux;
+        st.aux = c;
+        st.n_last = st.n_cur;
+        st.n_cur = appended;
+        if (appended == 0u || st.k >= max_k) break;
     }
     const unsigned ev = __reduce_add_sync(0xffffffffu, evals);
     if (lane == 0 && ev) atomicAdd(&s_evals, (unsigned long long)ev);
     __syncthreads();
+    if (tid == 0 && s_evals) atomicAdd(&ctrl->evals_list, s_evals);
+    if (blockIdx.x != 0 || failed) return;
+    // Every CTA holds the same state; the barriers order these writes after
+    // every CTA's reads of the control block.
+    // Whether the last pass changed the image.
+    const bool still = st.c_list ? st.n_cur != 0u : __ldcg(&ctrl->n_diff) != 0;
+    unsigned k = st.k;
+    if (still && st.n_cur == 0u) {
+        // The image alternates between the two canvases.
+        if ((max_k - k) & 1u) st.cur = st.aux;
+        k = max_k;
+    } else if (!still) {
+        // The last pass changed nothing; when it made an empty D_t, neither did the one before it.
+        k -= !st.c_list && st.n_cur == 0u ? 2u : 1u;
+    }
+    if (kBatch && a.img_k && still)
+        for (int i = tid; i < a.nimg; i += kListThreads)
+            if (__ldcg(a.img_n + i) != 0) a.img_k[i] = k;
     if (tid == 0) {
-        if (s_evals) atomicAdd(&ctrl->evals_list, s_evals);
-        if (blockIdx.x == 0 && !failed) {
-            // Every CTA holds the same state; the barriers order these writes
-            // after every CTA's reads of the control block.
-            ctrl->k = k;
-            if (converged) ctrl->converged = 1u;
-            ctrl->cur = cur;
-            ctrl->aux = aux;
-            ctrl->work_launches += 1u;
-            ctrl->executed += (unsigned)passes;
-        }
+        ctrl->executed += (still ? k : st.k) - k0;
+        ctrl->k = k;
+        if (!still) ctrl->converged = 1u;
+        ctrl->aux = 3u - st.cur - (3u - s_cur - s_aux);  // the other canvas of the pair
+        ctrl->cur = st.cur;
+        ctrl->work_launches += 1u;
     }
 }
 

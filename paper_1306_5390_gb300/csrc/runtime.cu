@@ -75,7 +75,7 @@ struct hgrms_ctx {
     size_t host_desc_cap = 0;
     int* tile_img = nullptr;
     size_t tile_cap = 0;
-    unsigned* img_k = nullptr;
+    unsigned* img_k = nullptr;  // img_k_cap k's, then as many counts of changed pixels (PassArgs::img_n)
     unsigned* host_img_k = nullptr;
     size_t img_k_cap = 0;
     std::vector<hg::ImgDesc> table_cache;  // what d_desc and tile_img hold now
@@ -436,7 +436,7 @@ int ensure_table(hgrms_ctx* h, size_t n, size_t tiles, bool per_image_k) {
         h->img_k = nullptr;
         h->host_img_k = nullptr;
         h->img_k_cap = 0;
-        HG_TRY(h, cudaMalloc(&h->img_k, n * sizeof(unsigned)));
+        HG_TRY(h, cudaMalloc(&h->img_k, 2 * n * sizeof(unsigned)));
         HG_TRY(h, cudaMallocHost(&h->host_img_k, n * sizeof(unsigned)));
         h->img_k_cap = n;
     }
@@ -709,6 +709,7 @@ int run_hybrid(hgrms_ctx* h, const BatchImg* im, int n, int alpha, int beta, int
     a.tile_img = h->tile_img;
     a.bm_total = bm_total;
     a.img_k = per_image_k ? h->img_k : nullptr;
+    a.img_n = per_image_k ? reinterpret_cast<int*>(h->img_k + h->img_k_cap) : nullptr;
     a.ntiles = (int)tiles_total;
     a.hybrid = 1;
     a.tile_eval_max = eval_max;
@@ -773,7 +774,7 @@ int run_hybrid(hgrms_ctx* h, const BatchImg* im, int n, int alpha, int beta, int
         HG_TRY(h, hg::launch_ctrl_init(h->ctrl, (unsigned)max_k, s));
         HG_TRY(h, cudaMemsetAsync(h->bitmaps, 0, 4 * (size_t)bm_total * sizeof(uint32_t), s));
         HG_TRY(h, cudaMemsetAsync(h->bar, 0, sizeof(hg::GridBar), s));
-        if (per_image_k) HG_TRY(h, cudaMemsetAsync(h->img_k, 0, (size_t)n * sizeof(unsigned), s));
+        if (per_image_k) HG_TRY(h, cudaMemsetAsync(h->img_k, 0, (h->img_k_cap + (size_t)n) * sizeof(unsigned), s));
         for (int i = 0; i < launches; ++i) {
             if (timed) HG_TRY(h, record(h->events[2 * i]));
             if (i < fused_launches) {

@@ -1,0 +1,174 @@
+"""The list passes' rules: which pixels a pass evaluates, when the lists
+change from C_t (pixels that differ from the previous pass's image) to D_t
+(pixels that differ from the image two passes back), and how k and the
+converged flag follow from the counts.
+
+CPU: the rules restated in numpy on top of the oracle's single passes, from
+every pass on, against the oracle's own iteration - bytes, k and converged
+flag are whole numbers, so equality.  GPU: the calls that reach each branch
+(one CTA alone, its hand-back to the grid when a list grows, the switch from C
+to D, empty D lists with pixels still alternating, capped lists, per-image k)
+against the oracle, tolerance zero.
+"""
+import numpy as np
+import pytest
+
+from paper_1306_5390_gb300 import synth
+
+
+def dilate(m, b):
+    rows, cols = m.shape
+    out = np.zeros_like(m)
+    for dy in range(-b, b + 1):
+        for dx in range(-b, b + 1):
+            ys, yd = max(0, -dy), max(0, dy)
+            xs, xd = max(0, -dx), max(0, dx)
+            if rows > abs(dy) and cols > abs(dx):
+                out[yd:rows - ys, xd:cols - xs] |= m[ys:rows - yd, xs:cols - xd]
+    return out
+
+
+def list_passes(oracle_mod, cur, aux, k, alpha, beta, max_k, c_first_below, solo):
+    """The loop from I_k = cur and I_(k-1) = aux on: (image, k, converged).
+    c_first_below: the first pass makes C when k is below it; solo: lists of at
+    most that many pixels are left to the passes that always make D."""
+    rows, cols = cur.shape
+    inner = np.zeros((rows, cols), dtype=bool)
+    if rows > 2 * beta and cols > 2 * beta:
+        inner[beta:rows - beta, beta:cols - beta] = True
+    listed, c_list, before, k0, N = cur != aux, True, 0, k, 0
+    while True:
+        n = int(listed.sum())
+        make_c = n > solo and c_list and (k0 < c_first_below if before == 0 else n * 5 < before * 3)
+        ev = dilate(listed, beta) & inner
+        new, _ = oracle_mod.one_pass(cur, alpha, beta)
+        out = np.where(ev, new, aux)  # a pixel that is not evaluated keeps what the output holds
+        now, was = ev & (out != cur), ev & (cur != aux)
+        if not make_c:
+            N += int(now.sum()) - (0 if c_list else int(was.sum()))
+        listed = ev & (out != (cur if make_c else aux))
+        cur, aux, before, c_list, k = out, cur, n, make_c, k + 1
+        if not listed.any() or k >= max_k:
+            break
+    empty = not listed.any()
+    still = (not empty) if c_list else N != 0
+    if still and empty:
+        return (aux if (max_k - k) % 2 else cur), max_k, False
+    if not still:
+        return cur, k - (2 if empty and not c_list else 1), True
+    return cur, k, False
+
+
+@pytest.mark.parametrize("beta", [1, 2, 3])
+def test_rules_give_the_oracles_iteration(oracle_mod, beta):
+    rng = np.random.default_rng(5390 + beta)
+    seen = set()
+    for trial in range(60):
+        rows, cols = (int(v) for v in rng.integers(2 * beta + 1, 2 * beta + 22, size=2))
+        alpha = int(rng.choice([0, 1, 5, 10, 60]))
+        kind = trial % 3
+        if kind == 0:
+            img = synth.noisy_image(rows, cols, float(rng.uniform(0.02, 0.7)), 100 * trial + beta)[1]
+        elif kind == 1:
+            img = synth.random_image(rows, cols, trial, levels=(0, 90, 100, 255))
+        else:
+            img = np.full((rows, cols), 100, np.uint8)
+            img[rows // 2, cols // 2] = 180
+        max_k = int(rng.choice([2, 3, 4, 9, 10, 33]))
+        ref, k_ref, c_ref = oracle_mod.denoise(img, alpha, beta, max_k)
+        aux, cur = img, img
+        for k0 in range(1, min(k_ref, max_k - 1) + 1):
+            aux, cur = cur, oracle_mod.one_pass(cur, alpha, beta)[0]
+            for below, solo in ((0, 0), (99, 0), (99, 3)):
+                out, k, c = list_passes(oracle_mod, cur, aux, k0, alpha, beta, max_k, below, solo)
+                assert (k, c) == (k_ref, c_ref) and np.array_equal(out, ref), (trial, rows, cols, alpha, max_k, k0,
+                                                                               below, solo, k, k_ref)
+            seen.add((bool(c_ref), k_ref == max_k))
+    assert {(True, False), (False, True)} <= seen
+
+
+@pytest.fixture(scope="module")
+def torch_cuda():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    return torch
+
+
+@pytest.fixture(scope="module")
+def den(torch_cuda):
+    from paper_1306_5390_gb300 import build, hgrms
+    build.build()
+    d = hgrms.Denoiser(0)
+    yield d
+    d.close()
+
+
+def single_dot(rows, cols):
+    img = np.full((rows, cols), 100, np.uint8)
+    img[rows // 2, cols // 3] = 201
+    return img
+
+
+# (image, alpha, beta, max_k, passes per launch, list capacity)
+CASES = [
+    ("dot", 0, 1, 60, 1, 0),     # spreads without end: one CTA, then the grid
+    ("dot", 0, 2, 41, 1, 0),
+    ("dot", 0, 7, 6, 1, 0),
+    ("dot", 0, 1, 60, 1, 300),   # ... and past the list's capacity
+    ("few", 10, 1, 9, 8, 0),     # one list pass
+    ("few", 10, 1, 10, 8, 0),
+    ("few", 10, 1, 33, 8, 0),
+    ("few", 10, 3, 33, 1, 0),
+    ("many", 10, 1, 31, 1, 0),   # both parities of the passes left over
+    ("many", 10, 1, 32, 1, 0),
+    ("many", 10, 2, 32, 2, 0),
+    ("many", 10, 2, 33, 4, 0),
+    ("many", 10, 3, 32, 1, 0),
+    ("many", 5, 1, 40, 1, 50),
+    ("many", 10, 2, 2000, 4, 0),
+    ("low", 10, 5, 32, 1, 0),    # dies out: C lists to the end
+    ("low", 10, 7, 32, 1, 0),
+]
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("name,alpha,beta,max_k,passes,cap", CASES)
+def test_list_pass_branches(oracle_mod, den, torch_cuda, name, alpha, beta, max_k, passes, cap):
+    from paper_1306_5390_gb300 import hgrms
+    img = {"dot": lambda: single_dot(151, 263),
+           "few": lambda: synth.noisy_image(200, 300, 0.2, 71)[1],
+           "many": lambda: synth.noisy_image(403, 517, 0.5, 72)[1],
+           "low": lambda: synth.noisy_image(500, 301, 0.02, 73)[1]}[name]()
+    den.set_option(hgrms.HGRMS_OPT_PASSES, passes)
+    den.set_option(hgrms.HGRMS_OPT_LIST_CAP, cap)
+    try:
+        t = torch_cuda.from_numpy(img.copy()).cuda()
+        k = den.denoise(t, alpha, beta, max_k)
+        conv = den.converged()
+    finally:
+        den.set_option(hgrms.HGRMS_OPT_PASSES, 0)
+        den.set_option(hgrms.HGRMS_OPT_LIST_CAP, 0)
+    ref, k_ref, c_ref = oracle_mod.denoise(img, alpha, beta, max_k)
+    assert (k, conv) == (k_ref, c_ref)
+    assert np.array_equal(t.cpu().numpy(), ref)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("beta,max_k,cap", [(1, 9, 0), (1, 12, 0), (1, 33, 0), (2, 6, 0), (2, 32, 0), (3, 17, 0), (1, 33, 200)])
+def test_batch_k_of_images_that_stop_at_different_passes(oracle_mod, den, torch_cuda, beta, max_k, cap):
+    from paper_1306_5390_gb300 import hgrms
+    imgs = [synth.noisy_image(40 + 23 * i, 300 - 17 * i, 0.05 * i, 900 + i)[1] for i in range(12)]
+    imgs.append(single_dot(30, 30))
+    den.set_option(hgrms.HGRMS_OPT_PASSES, 1 if max_k < 9 else 0)
+    den.set_option(hgrms.HGRMS_OPT_LIST_CAP, cap)
+    try:
+        ts = [torch_cuda.from_numpy(im.copy()).cuda() for im in imgs]
+        ks = den.denoise_batch(ts, 10, beta, max_k)
+    finally:
+        den.set_option(hgrms.HGRMS_OPT_PASSES, 0)
+        den.set_option(hgrms.HGRMS_OPT_LIST_CAP, 0)
+    for i, (im, t, k) in enumerate(zip(imgs, ts, ks)):
+        ref, k_ref, c_ref = oracle_mod.denoise(im, 10, beta, max_k)
+        assert k == k_ref and (k < max_k) == c_ref, (i, k, k_ref)
+        assert np.array_equal(t.cpu().numpy(), ref), i
