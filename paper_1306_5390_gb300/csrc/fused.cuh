@@ -158,6 +158,12 @@ __device__ __forceinline__ uint32_t h2_to_bytes(uint32_t a, uint32_t b) {
     return __byte_perm(ab, bb, 0x6420);
 }
 
+// Bit j: byte j of d is not zero.
+__device__ __forceinline__ uint32_t changed_bytes(uint32_t d) {
+    const uint32_t m = ((((d & 0x7F7F7F7Fu) + 0x7F7F7F7Fu) | d) >> 7) & 0x01010101u;
+    return (m * 0x01020408u >> 24) & 0xFu;
+}
+
 // One tile row as seen by one segment: fp16 pairs starting at pixel offsets
 // -B .. 6+B relative to the segment's first pixel.
 template <int B>
@@ -1192,12 +1198,25 @@ fused_kernel(PassArgs a) {
         const uint32_t* pen = (np & 1) ? buf0 : buf1;  // I_(np-1) (the loaded tile when np == 1)
 
         // Core -> canvas bytes (and I_(np-1) -> the third canvas when asked).
+        // Hybrid schedule: the pixels where the two differ are the last
+        // pass's changes, this launch's change set.  They are found here, from
+        // the words in hand, so the set is complete however many there are
+        // (the passes' own lists hold at most kListCap; a tile that overflowed
+        // its list used to make the next pass evaluate every pixel of every
+        // image).
+        constexpr int CH = G::TW / 16;
+        constexpr int kIt = (G::TH * CH + G::kThreads - 1) / G::kThreads;
+        uint32_t chm[kIt];  // changed pixels of this thread's chunks (bit: column)
+        int nch = 0;
         {
             const long long off = (long long)(kPadY + y0) * pitch + kPadX + x0;
             uint8_t* base = dst + off;
             uint8_t* base_prev = a.canvas[third] + coff + off;
-            constexpr int CH = G::TW / 16;
-            for (int i = tid; i < G::TH * CH; i += G::kThreads) {
+#pragma unroll
+            for (int it = 0; it < kIt; ++it) {
+                const int i = tid + it * G::kThreads;
+                chm[it] = 0u;
+                if (i >= G::TH * CH) continue;
                 const int r = i / CH, cc = i - r * CH;
                 const int so = (G::H + r) * G::SWW + kPadX / 2 + cc * 8;
                 const uint4* s = reinterpret_cast<const uint4*>(fin + so);
@@ -1211,47 +1230,48 @@ fused_kernel(PassArgs a) {
                 if (a.write_prev) {
                     const uint4* s2 = reinterpret_cast<const uint4*>(pen + so);
                     const uint4 p2 = s2[0], q2 = s2[1];
-                    o.x = h2_to_bytes(p2.x, p2.y);
-                    o.y = h2_to_bytes(p2.z, p2.w);
-                    o.z = h2_to_bytes(q2.x, q2.y);
-                    o.w = h2_to_bytes(q2.z, q2.w);
-                    *reinterpret_cast<uint4*>(base_prev + (long long)r * pitch + cc * 16) = o;
+                    uint4 o2;
+                    o2.x = h2_to_bytes(p2.x, p2.y);
+                    o2.y = h2_to_bytes(p2.z, p2.w);
+                    o2.z = h2_to_bytes(q2.x, q2.y);
+                    o2.w = h2_to_bytes(q2.z, q2.w);
+                    *reinterpret_cast<uint4*>(base_prev + (long long)r * pitch + cc * 16) = o2;
+                    // Positions outside the image never change, so a chunk
+                    // with changes lies in the image's bitmap row; its 16 bits
+                    // are written whole (the bitmap is clear before).
+                    chm[it] = changed_bytes(o.x ^ o2.x) | changed_bytes(o.y ^ o2.y) << 4 |
+                              changed_bytes(o.z ^ o2.z) << 8 | changed_bytes(o.w ^ o2.w) << 12;
+                    if (a.hybrid && chm[it]) {
+                        nch += __popc(chm[it]);
+                        reinterpret_cast<uint16_t*>(a.bitmaps[set_out] + bm_off + (size_t)(y0 + r) * bm_words)[(x0 >> 4) + cc] =
+                            (uint16_t)chm[it];
+                    }
                 }
+            }
+        }
+        if (a.hybrid) {
+            // Its list: one global atomic per tile.
+            int* s_sel = s_cnt + 4;  // [0]: changed pixels, [1]: global base
+            int wtot;
+            int pos = warp_excl_scan(lane, nch, &wtot);
+            int wbase = 0;
+            if (lane == 0 && wtot) wbase = atomicAdd(&s_sel[0], wtot);
+            pos += __shfl_sync(0xffffffffu, wbase, 0);
+            __syncthreads();
+            if (tid == 0) s_sel[1] = s_sel[0] ? (int)atomicAdd(&ctrl->list_n[set_out], (unsigned)s_sel[0]) : 0;
+            __syncthreads();
+            unsigned gpos = (unsigned)s_sel[1] + (unsigned)pos;
+            uint32_t* glist = a.lists[set_out];
+#pragma unroll
+            for (int it = 0; it < kIt; ++it) {
+                const int i = tid + it * G::kThreads;
+                const int r = i / CH, cc = i - r * CH;
+                for (uint32_t m = chm[it]; m; m &= m - 1u, ++gpos)
+                    if (gpos < a.list_cap) glist[gpos] = pack_entry(img, y0 + r, x0 + cc * 16 + __ffs(m) - 1, a.xb, a.yb);
             }
         }
         const int nlast = s_cnt[(np - 1) % 3];
         const uint16_t* last = lists + ((np - 1) & 1) * G::kListCap;
-        // The last pass's changed core pixels -> this launch's change set
-        // (one global atomic per tile); an overflowed tile list marks the
-        // set as overflowed, so the next pass evaluates every pixel.
-        if (a.hybrid) {
-            uint32_t* glist = a.lists[set_out];
-            unsigned* gn = &ctrl->list_n[set_out];
-            uint32_t* gbm = a.bitmaps[set_out];
-            int* s_sel = s_cnt + 4;  // [0]: core entries, [1]: global base
-            if (nlast <= G::kListCap) {
-                // Compact the core entries to the front of `cand` (free now).
-                uint32_t* sel = reinterpret_cast<uint32_t*>(smem + G::kCandOff);
-                for (int i = tid; i < nlast; i += G::kThreads) {
-                    const int q = last[i];
-                    const int y = q / G::SW, x = q - y * G::SW;
-                    const int gy = y0 + y - G::H, gx = x0 + x - kPadX;
-                    if (in_core_px(y, x, G::H, G::TH, G::TW) && gy < rows && gx < cols) {
-                        sel[atomicAdd(&s_sel[0], 1)] = pack_entry(img, gy, gx, a.xb, a.yb);
-                        atomicOr(gbm + bm_off + (size_t)gy * bm_words + (gx >> 5), 1u << (gx & 31));
-                    }
-                }
-                __syncthreads();
-                const int nsel = s_sel[0];
-                if (tid == 0) s_sel[1] = nsel ? (int)atomicAdd(gn, (unsigned)nsel) : 0;
-                __syncthreads();
-                const unsigned gbase = (unsigned)s_sel[1];
-                for (int i = tid; i < nsel; i += G::kThreads)
-                    if (gbase + i < a.list_cap) glist[gbase + i] = sel[i];
-            } else if (tid == 0) {
-                atomicAdd(gn, a.list_cap + 1u);  // overflow: the next pass evaluates every pixel
-            }
-        }
         // The last pass's changed core pixels -> this launch's map (all core
         // pixels when the list overflowed: a superset is always safe).
         if (use_maps) {

@@ -157,11 +157,17 @@ namespace {
 
 // Hybrid schedule: fused launches after the first (each runs only when the
 // previous one left many changed pixels; a launch that does not run still
-// costs a few microseconds).  Default: for beta 1 (T = 8, the cheapest fused
-// pass) up to 3 of them, when a list pass would evaluate more than 2.5 % of
-// the pixels (measured on GB300: list passes stay faster below that); none
-// for wider windows, whose fused passes cost more than list passes even on
-// dense change sets.  With HGRMS_OPT_RELAUNCH_PPM set, up to 8 for any beta.
+// costs 4 to 6 us).  With alpha >= 2 the list passes take over after the first
+// launch whatever it left, because their lists shrink by about half per pass
+// (list.cu): 128 images of 128..2048 pixels a side, 5..70 % impulses, 3.39 ms
+// a call without relaunches against 3.75 ms with one and 5.14 ms with three;
+// 8192 x 8192 at 70 % 2.18 against 2.55 and 3.77 ms; 2048 x 2048 at 50 % 0.349
+// against 0.366 and 0.396 ms.  With alpha 0 every interior pixel is replaced
+// in every pass and no list shrinks, and with alpha 1 the lists of a noise
+// image shrink slowly (18 % of the pixels after 8 passes): there, for beta 1
+// (T = 8, the cheapest fused pass) and large calls, up to 3 of them run when a
+// list pass would evaluate more than 2.5 % of the pixels.  With
+// HGRMS_OPT_RELAUNCH_PPM set, up to 8 for any alpha and beta.
 constexpr int kDefaultRelaunches = 3;
 // Calls of at least this many pixels use the 128-row tiles (where compiled
 // and they compute fewer rows): measured faster on 8192 x 8192 and on the
@@ -171,8 +177,8 @@ constexpr long long kTallMinPixels = 32ll << 20;
 constexpr long long kRelaunchMinPixels = 4ll << 20;
 constexpr size_t kMaxGraphs = 8;  // captured graphs kept per handle (HGRMS_OPT_GRAPH)
 constexpr int kMaxRelaunches = 8;
-long long default_relaunch_ppm(int beta) {
-    return beta == 1 ? 25000 : 1000000;
+long long default_relaunch_ppm(int alpha, int beta) {
+    return beta == 1 && alpha <= 1 ? 25000 : 1000000;
 }
 
 using hg::default_passes;
@@ -727,11 +733,10 @@ int run_hybrid(hgrms_ctx* h, const BatchImg* im, int n, int alpha, int beta, int
     a.bar_extra = h->opt_wait_test > 0 ? 1u : 0u;
     a.bar_spins = (unsigned)h->opt_wait_test;
     const bool user_ppm = h->opt_relaunch_ppm > 0;
-    const long long ppm = user_ppm ? h->opt_relaunch_ppm : default_relaunch_ppm(beta);
+    const long long ppm = user_ppm ? h->opt_relaunch_ppm : default_relaunch_ppm(alpha, beta);
     a.relaunch_evals = ppm >= 1000000 ? (1ll << 62) : px_total / 1000000 * ppm + px_total % 1000000 * ppm / 1000000;
     // Built-in: relaunch slots only for calls of at least kRelaunchMinPixels
-    // (below that the list passes are cheap, and each slot a launch that
-    // usually finds nothing to do: ~5 us of a ~100 us call on 256 x 256).
+    // (below that the list passes are cheap).
     int relaunches = ppm >= 1000000 ? 0
                                     : (user_ppm ? kMaxRelaunches
                                                 : (px_total >= kRelaunchMinPixels ? kDefaultRelaunches : 0));

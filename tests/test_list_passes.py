@@ -28,10 +28,9 @@ def dilate(m, b):
     return out
 
 
-def list_passes(oracle_mod, cur, aux, k, alpha, beta, max_k, c_first_below, solo):
+def list_passes(oracle_mod, cur, aux, k, alpha, beta, max_k, c_first_below):
     """The loop from I_k = cur and I_(k-1) = aux on: (image, k, converged).
-    c_first_below: the first pass makes C when k is below it; solo: lists of at
-    most that many pixels are left to the passes that always make D."""
+    c_first_below: the first pass makes C when k is below it."""
     rows, cols = cur.shape
     inner = np.zeros((rows, cols), dtype=bool)
     if rows > 2 * beta and cols > 2 * beta:
@@ -39,7 +38,7 @@ def list_passes(oracle_mod, cur, aux, k, alpha, beta, max_k, c_first_below, solo
     listed, c_list, before, k0, N = cur != aux, True, 0, k, 0
     while True:
         n = int(listed.sum())
-        make_c = n > solo and c_list and (k0 < c_first_below if before == 0 else n * 5 < before * 3)
+        make_c = c_list and (k0 < c_first_below if before == 0 else n * 5 < before * 3)
         ev = dilate(listed, beta) & inner
         new, _ = oracle_mod.one_pass(cur, alpha, beta)
         out = np.where(ev, new, aux)  # a pixel that is not evaluated keeps what the output holds
@@ -79,10 +78,10 @@ def test_rules_give_the_oracles_iteration(oracle_mod, beta):
         aux, cur = img, img
         for k0 in range(1, min(k_ref, max_k - 1) + 1):
             aux, cur = cur, oracle_mod.one_pass(cur, alpha, beta)[0]
-            for below, solo in ((0, 0), (99, 0), (99, 3)):
-                out, k, c = list_passes(oracle_mod, cur, aux, k0, alpha, beta, max_k, below, solo)
+            for below in (0, 99):
+                out, k, c = list_passes(oracle_mod, cur, aux, k0, alpha, beta, max_k, below)
                 assert (k, c) == (k_ref, c_ref) and np.array_equal(out, ref), (trial, rows, cols, alpha, max_k, k0,
-                                                                               below, solo, k, k_ref)
+                                                                               below, k, k_ref)
             seen.add((bool(c_ref), k_ref == max_k))
     assert {(True, False), (False, True)} <= seen
 
@@ -172,3 +171,39 @@ def test_batch_k_of_images_that_stop_at_different_passes(oracle_mod, den, torch_
         ref, k_ref, c_ref = oracle_mod.denoise(im, 10, beta, max_k)
         assert k == k_ref and (k < max_k) == c_ref, (i, k, k_ref)
         assert np.array_equal(t.cpu().numpy(), ref), i
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("cols", [225, 239, 240, 241, 255, 257, 480])
+@pytest.mark.parametrize("beta", [1, 2, 3])
+def test_change_set_of_a_dense_last_pass(oracle_mod, den, torch_cuda, beta, cols):
+    """One fused pass that leaves more changes per tile than the passes' own
+    lists hold, at widths around the ends of tiles and bitmap words; then list
+    passes."""
+    from paper_1306_5390_gb300 import hgrms
+    img = synth.random_image(131, cols, 40 + cols)
+    assert oracle_mod.one_pass(img, 2, beta)[1] > 2 * 1024
+    ref, k_ref, c_ref = oracle_mod.denoise(img, 2, beta, 12)
+    den.set_option(hgrms.HGRMS_OPT_PASSES, 1)
+    den.set_option(hgrms.HGRMS_OPT_LIST_CAP, 1 << 20)
+    try:
+        t = torch_cuda.from_numpy(img.copy()).cuda()
+        k = den.denoise(t, 2, beta, 12)
+    finally:
+        den.set_option(hgrms.HGRMS_OPT_PASSES, 0)
+        den.set_option(hgrms.HGRMS_OPT_LIST_CAP, 0)
+    assert (k, den.converged()) == (k_ref, c_ref)
+    assert np.array_equal(t.cpu().numpy(), ref)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("alpha", [0, 1, 2])
+def test_relaunch_rule_of_large_calls(oracle_mod, den, torch_cuda, alpha):
+    """Calls of 4 Mi pixels: alpha 0 and 1 run further fused launches, others list passes only."""
+    img = synth.noisy_image(2051, 2049, 0.3, 74)[1]
+    t = torch_cuda.from_numpy(img.copy()).cuda()
+    k = den.denoise(t, alpha, 1, 18)
+    ref, k_ref, c_ref = oracle_mod.denoise(img, alpha, 1, 18)
+    assert den.stats()["launches"] == (4 if alpha <= 1 else 2)
+    assert (k, den.converged()) == (k_ref, c_ref)
+    assert np.array_equal(t.cpu().numpy(), ref)
