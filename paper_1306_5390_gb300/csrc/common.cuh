@@ -47,9 +47,10 @@ struct Ctrl {
     unsigned long long evals_fused;
     unsigned long long evals_list;
     // List-pass launch: pixels changed by the last pass it ran, and the state
-    // that the passes of one CTA alone leave to the others (k, list length).
+    // that the passes of one CTA alone leave to the others (k, list length,
+    // length of the list before, or ~0 when the list is a D_t).
     int n_diff;
-    unsigned solo_k, solo_n;
+    unsigned solo_k, solo_n, solo_before;
 };
 
 // Grid barrier of the list-pass loop: two 64-bit counters on their own

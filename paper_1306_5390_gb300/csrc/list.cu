@@ -287,7 +287,13 @@ struct LoopState {
     unsigned cur, aux;  // canvases of I_t and I_(t-1)
     unsigned n_cur;     // entries of the list the next pass reads
     unsigned n_last;    // entries of the list before it (its bitmap is cleared by the next pass)
+    unsigned n_before;  // entries of the list that the last pass read (0: no pass yet)
     bool c_list;        // the next pass reads C_t (else D_t)
+    // Whether the next pass, from a list of n entries, makes C (see the header; k0: passes before this launch).
+    __device__ __forceinline__ bool make_c(unsigned n, unsigned k0) const {
+        return c_list && (n_before == 0u ? k0 < kDirectD
+                                         : (unsigned long long)n * 5u < (unsigned long long)n_before * 3u);
+    }
 };
 
 // Passes run by CTA 0 alone, from a list of st.n_cur <= kSoloEvals / P
@@ -302,7 +308,7 @@ struct LoopState {
 // counters; dn accumulates this thread's share of the change of N.
 template <int B, bool kBatch>
 __device__ __forceinline__ void solo_passes(const PassArgs& a, const ImgDesc& one, const int base, const int xb,
-                                            const int yb, const unsigned max_k, LoopState& st, uint32_t* lists,
+                                            const int yb, const unsigned max_k, const unsigned k0, LoopState& st, uint32_t* lists,
                                             uint32_t* hash, unsigned* s_n, unsigned& evals, int& dn) {
     constexpr int W = 2 * B + 1, P = W * W, NW = (W + 3) / 4;
     const int tid = threadIdx.x;
@@ -334,6 +340,7 @@ __device__ __forceinline__ void solo_passes(const PassArgs& a, const ImgDesc& on
         const uint8_t* in_arena = a.canvas[st.cur];
         uint8_t* out_arena = a.canvas[st.aux];
         const int ntask = (int)n * P;
+        const bool make_c = st.make_c(n, k0);
         for (int i = tid; i < ntask; i += kListThreads) {
             const int e = i / P, o = i - e * P;
             unsigned img;
@@ -364,12 +371,10 @@ __device__ __forceinline__ void solo_passes(const PassArgs& a, const ImgDesc& on
             ++evals;
             const int ip = (int)((win[B][B / 4] >> (8 * (B % 4))) & 0xffu);
             const int nv = eval_window<B>(win, a.alpha);
-            if (nv != was) {
-                out_arena[off] = (uint8_t)nv;
-                next[atomicAdd(nn, 1u)] = key;
-            }
+            if (nv != was) out_arena[off] = (uint8_t)nv;
+            if (nv != (make_c ? ip : was)) next[atomicAdd(nn, 1u)] = key;
             const int now = nv != ip ? 1 : 0, before = ip != was ? 1 : 0;
-            const int delta = now - (st.c_list ? 0 : before);
+            const int delta = (make_c ? 0 : now) - (st.c_list ? 0 : before);
             dn += delta;
             if (kBatch && a.img_k) {
                 if (delta) atomicAdd(a.img_n + img, delta);
@@ -377,9 +382,10 @@ __device__ __forceinline__ void solo_passes(const PassArgs& a, const ImgDesc& on
             }
         }
         __syncthreads();
+        st.n_before = n;
         n = *nn;
         ++st.k;
-        st.c_list = false;
+        st.c_list = make_c;
         const unsigned c = st.cur;
         st.cur = st.aux;
         st.aux = c;
@@ -450,7 +456,7 @@ __global__ void __launch_bounds__(kListThreads, 2) list_loop_kernel(PassArgs a) 
     st.cur = s_cur;
     st.aux = s_aux;
     st.c_list = true;
-    unsigned n_before = 0;  // entries of the list that the previous pass read
+    st.n_before = 0u;
     unsigned gen = 0u;                // barriers completed; the barrier struct is zeroed at the start of every call
     unsigned prev_hi[2] = {0u, 0u};  // thread 0: counts seen at the last use of each barrier counter
     const int base = (int)s_base;
@@ -494,7 +500,7 @@ __global__ void __launch_bounds__(kListThreads, 2) list_loop_kernel(PassArgs a) 
         if (st.n_cur <= (unsigned)(kSoloEvals / P) && st.n_cur <= a.list_cap && st.n_last <= kSoloClear &&
             st.n_last <= a.list_cap) {
             if (blockIdx.x == 0) {
-                solo_passes<B, kBatch>(a, one, base, xb, yb, max_k, st, stage_all, s_queue, s_solo_n, evals, dn);
+                solo_passes<B, kBatch>(a, one, base, xb, yb, max_k, k0, st, stage_all, s_queue, s_solo_n, evals, dn);
                 dn = __reduce_add_sync(0xffffffffu, dn);
                 if (lane == 0 && dn) atomicAdd(&s_dn, dn);
                 __syncthreads();
@@ -504,6 +510,7 @@ __global__ void __launch_bounds__(kListThreads, 2) list_loop_kernel(PassArgs a) 
                     s_dn = 0;
                     ctrl->solo_k = st.k;
                     ctrl->solo_n = st.n_cur;
+                    ctrl->solo_before = st.c_list ? st.n_before : 0xffffffffu;
                 }
             }
             unsigned zero = 0;
@@ -515,13 +522,15 @@ __global__ void __launch_bounds__(kListThreads, 2) list_loop_kernel(PassArgs a) 
                 if (tid == 0) {
                     s_k = __ldcg(&ctrl->solo_k);
                     s_n = __ldcg(&ctrl->solo_n);
+                    s_nclr = __ldcg(&ctrl->solo_before);
                 }
                 __syncthreads();
                 const unsigned ran = s_k - st.k;
                 st.k = s_k;
                 st.n_cur = s_n;
                 st.n_last = 0u;
-                st.c_list = false;
+                st.n_before = s_nclr;
+                st.c_list = s_nclr != 0xffffffffu;
                 if (ran & 1u) {
                     const unsigned c = st.cur;
                     st.cur = st.aux;
@@ -539,8 +548,7 @@ __global__ void __launch_bounds__(kListThreads, 2) list_loop_kernel(PassArgs a) 
         uint32_t* next = a.lists[so];
         uint32_t* bm_next = a.bitmaps[so];
         unsigned* nnext = &ctrl->list_n[so];
-        // Which list this pass makes (see the header).
-        const bool make_c = st.c_list && (n_before == 0u ? k0 < kDirectD : (unsigned long long)st.n_cur * 5u < (unsigned long long)n_before * 3u);
+        const bool make_c = st.make_c(st.n_cur, k0);
         // N is needed from the first D_t on: the pass that makes it counts the
         // pixels it changes, the later ones the differences.
         const int add = make_c ? 0 : 1, sub = st.c_list ? 0 : 1;
@@ -851,7 +859,7 @@ __global__ void __launch_bounds__(kListThreads, 2) list_loop_kernel(PassArgs a) 
         ++st.t;
         ++st.k;
         st.c_list = make_c;
-        n_before = st.n_cur;
+        st.n_before = st.n_cur;
         const unsigned c = st.cur;
         st.cur = st.aux;
         st.aux = c;
