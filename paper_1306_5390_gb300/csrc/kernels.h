@@ -21,16 +21,27 @@ const FusedEntry* find_fused(int beta, int T, int rn = 64);
 int default_passes(int beta);
 
 cudaError_t launch_plain(int beta, const PassArgs& a, cudaStream_t s);
-cudaError_t launch_ctrl_init(Ctrl* c, unsigned max_k, cudaStream_t s);
+// Clear a call's control block, bitmaps (n16 16-byte words), barrier and per-image counts (nk words).
+cudaError_t launch_call_init(Ctrl* c, unsigned max_k, uint32_t* bm, long long n16, GridBar* bar, unsigned* counts,
+                             long long nk, int sms, cudaStream_t s);
 cudaError_t launch_copy_in(const uint8_t* img, int rows, int cols, uint8_t* canvas, long long pitch,
                            int sms, cudaStream_t s);
-cudaError_t launch_copy_out(const Ctrl* c, uint8_t* const canvas[3], long long pitch, uint8_t* img, int rows,
-                            int cols, int sms, cudaStream_t s);
+// The end of a call (call_finish_kernel): images out and the results to the host.
+struct FinishArgs {
+    const Ctrl* ctrl;
+    const uint8_t* arena[3];
+    const ImgDesc* imgs;    // a batch: the image table (images without `user` are not written); null: one image
+    int nimg;
+    uint8_t* user;          // one image: where it goes
+    long long pitch;        // ... and its canvas pitch
+    int rows, cols;         // one image's size; a batch's largest rows and columns
+    int write;              // 0: images stay as they are
+    Ctrl* host_ctrl;        // page-locked copy of the control block, or null
+    const unsigned* img_k;  // a batch's per-image k
+    unsigned* host_img_k;   // ... and its page-locked copy, or null
+};
+cudaError_t launch_call_finish(const FinishArgs& a, int sms, cudaStream_t s);
 cudaError_t launch_list(int beta, const PassArgs& a, int sms, cudaStream_t s);
-// Batched forms (image table on the device; max_words = the largest image's
-// rows * cols / 4, rounded up, sizes the grid).
-cudaError_t launch_copy_out_batch(const Ctrl* c, uint8_t* const arena[3], const ImgDesc* imgs, int nimg,
-                                  long long max_words, int sms, cudaStream_t s);
 cudaError_t launch_tile_map(const ImgDesc* imgs, int nimg, int total_tiles, int* tile_img, cudaStream_t s);
 // out[i] = floor(sqrt(floor(sum[i] / flag[i]))) by the kernels' integer root mean square (rms_div).
 cudaError_t launch_rms(const int* sum, const int* flag, int* out, int n, cudaStream_t s);

@@ -130,11 +130,11 @@ extern "C" __attribute__((visibility("default"))) int hgrms_denoise_noalloc(uint
     a.list_ctas = 0;
 
     // The array keeps the previous call's contents: the control block is
-    // reset by ctrl_init and change map 0 (written by the first launch) is
+    // reset by the call's first launch and change map 0 (written by the first launch) is
     // cleared here; the launches clear the other maps themselves.  Canvas
     // bytes outside the image are never read by a pixel that can change.
     HG_NA_TRY(hg::launch_copy_in(img, rows, cols, a.canvas[0], pitch, sms, s));
-    HG_NA_TRY(hg::launch_ctrl_init(ctrl, (unsigned)max_k, s));
+    HG_NA_TRY(hg::launch_call_init(ctrl, (unsigned)max_k, nullptr, 0, nullptr, nullptr, 0, sms, s));
     HG_NA_TRY(cudaMemsetAsync(a.chg_maps, 0, map_bytes, s));
     // Launches after the call has converged return at once but still cost a
     // wave each, so they are queued in groups, and between groups the host
@@ -152,7 +152,16 @@ extern "C" __attribute__((visibility("default"))) int hgrms_denoise_noalloc(uint
             if (st[1] || st[0] >= (unsigned)max_k) break;
         }
     }
-    HG_NA_TRY(hg::launch_copy_out(ctrl, a.canvas, pitch, img, rows, cols, sms, s));
+    hg::FinishArgs fa = {};
+    fa.ctrl = ctrl;
+    for (int c = 0; c < 3; ++c) fa.arena[c] = a.canvas[c];
+    fa.nimg = 1;
+    fa.user = img;
+    fa.pitch = pitch;
+    fa.rows = rows;
+    fa.cols = cols;
+    fa.write = 1;
+    HG_NA_TRY(hg::launch_call_finish(fa, sms, s));
     unsigned k = 0;
     HG_NA_TRY(cudaMemcpyAsync(&k, &ctrl->k, sizeof(k), cudaMemcpyDeviceToHost, s));
     HG_NA_TRY(cudaStreamSynchronize(s));

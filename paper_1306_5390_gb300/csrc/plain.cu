@@ -1,5 +1,5 @@
-// Unfused one-pass kernel (one thread per pixel, global loads), canvas copy
-// kernels and the control-block initialiser.
+// Unfused one-pass kernel (one thread per pixel, global loads) and the kernels
+// that begin and end a call.
 //
 // The unfused kernel evaluates Algorithms 1 and 2 directly for each pixel:
 // card by gathering over the window (equal to the paper's scattered
@@ -7,6 +7,8 @@
 // symmetric), then flag / sum / replacement.  It is the straightforward GPU
 // form of the method, kept as a second, independent device path and as the
 // unfused point of comparison for the fused tile kernel.
+#include <algorithm>
+
 #include "common.cuh"
 #include "kernels.h"
 
@@ -83,33 +85,34 @@ cudaError_t launch_plain(int beta, const PassArgs& a, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-__global__ void ctrl_init_kernel(Ctrl* c, unsigned max_k) {
-    c->k = 0;
-    c->converged = 0;
-    c->cur = 0;
-    c->aux = 1;
-    c->max_k = max_k;
-    c->done = 0;
-    c->mask = 0;
-    c->work_launches = 0;
-    c->executed = 0;
-    for (int i = 0; i < 4; ++i) c->list_n[i] = 0;
-    c->error = 0;
-    c->evals_fused = 0;
-    c->evals_list = 0;
-    c->n_diff = 0;
-    c->fused_work = 0;
-    c->dense = 0;
-    c->tile_next[0] = 0;
-    c->tile_next[1] = 0;
+// Everything a call needs cleared, in one launch: the control block, the
+// change bitmaps (n16 16-byte words), the barrier and, for a batch, the
+// per-image counts (nk words).  (One kernel for the control block and a memset
+// for each of the others cost a call two to three launches more, ~1.5 us
+// each.)
+__global__ void call_init_kernel(Ctrl* __restrict__ c, unsigned max_k, uint4* __restrict__ bm, long long n16,
+                                 GridBar* __restrict__ bar, unsigned* __restrict__ counts, long long nk) {
+    const long long g = blockIdx.x * (long long)blockDim.x + threadIdx.x, gt = (long long)gridDim.x * blockDim.x;
+    if (g == 0) {
+        Ctrl z = {};
+        z.aux = 1;
+        z.max_k = max_k;
+        *c = z;
+        if (bar) bar->ctr[0].v = bar->ctr[1].v = 0ull;
+    }
+    for (long long i = g; i < nk; i += gt) counts[i] = 0u;
+    for (long long i = g; i < n16; i += gt) bm[i] = make_uint4(0u, 0u, 0u, 0u);
 }
 
-cudaError_t launch_ctrl_init(Ctrl* c, unsigned max_k, cudaStream_t s) {
-    ctrl_init_kernel<<<1, 1, 0, s>>>(c, max_k);
+cudaError_t launch_call_init(Ctrl* c, unsigned max_k, uint32_t* bm, long long n16, GridBar* bar, unsigned* counts,
+                             long long nk, int sms, cudaStream_t s) {
+    long long blocks = (std::max(n16, nk) + 1023) / 1024;  // four words a thread
+    blocks = std::min(std::max(blocks, 1ll), (long long)sms * 8);
+    call_init_kernel<<<(unsigned)blocks, 256, 0, s>>>(c, max_k, reinterpret_cast<uint4*>(bm), n16, bar, counts, nk);
     return cudaGetLastError();
 }
 
-// Dense user image (row r at img + r*cols) <-> canvas interior, in 16-byte
+// Dense user image (row r at img + r*cols) -> canvas interior, in 16-byte
 // row chunks; vector accesses when the user rows are 16-byte aligned.
 __global__ void copy_in_kernel(const uint8_t* __restrict__ img, int rows, int cols,
                                uint8_t* __restrict__ canvas, long long pitch, int vec) {
@@ -124,28 +127,6 @@ __global__ void copy_in_kernel(const uint8_t* __restrict__ img, int rows, int co
         const int n = min(16, cols - x);
         if (vec && n == 16) {
             *reinterpret_cast<uint4*>(d) = __ldg(reinterpret_cast<const uint4*>(s));
-        } else {
-            for (int b = 0; b < n; ++b) d[b] = s[b];
-        }
-    }
-}
-
-__global__ void copy_out_kernel(const Ctrl* __restrict__ c, const uint8_t* __restrict__ c0,
-                                const uint8_t* __restrict__ c1, const uint8_t* __restrict__ c2, long long pitch,
-                                uint8_t* __restrict__ img, int rows, int cols, int vec) {
-    const unsigned cur = __ldcg(&c->cur);
-    const uint8_t* canvas = cur == 0 ? c0 : (cur == 1 ? c1 : c2);
-    const long long chunks = (cols + 15) / 16;
-    const long long total = chunks * rows;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
-         i += (long long)gridDim.x * blockDim.x) {
-        const long long r = i / chunks;
-        const int x = (int)(i - r * chunks) * 16;
-        const uint8_t* s = canvas + (kPadY + r) * pitch + kPadX + x;
-        uint8_t* d = img + r * cols + x;
-        const int n = min(16, cols - x);
-        if (vec && n == 16) {
-            *reinterpret_cast<uint4*>(d) = *reinterpret_cast<const uint4*>(s);
         } else {
             for (int b = 0; b < n; ++b) d[b] = s[b];
         }
@@ -168,57 +149,91 @@ cudaError_t launch_copy_in(const uint8_t* img, int rows, int cols, uint8_t* canv
     return cudaGetLastError();
 }
 
-cudaError_t launch_copy_out(const Ctrl* c, uint8_t* const canvas[3], long long pitch, uint8_t* img, int rows,
-                            int cols, int sms, cudaStream_t s) {
-    const int vec = (cols % 16 == 0) && ((reinterpret_cast<uintptr_t>(img) & 15u) == 0);
-    copy_out_kernel<<<copy_grid(rows, cols, sms), 256, 0, s>>>(c, canvas[0], canvas[1], canvas[2], pitch, img,
-                                                               rows, cols, vec);
-    return cudaGetLastError();
+// The end of a call: canvas `cur` -> the caller's dense images, and the
+// control block (and a batch's per-image k) -> page-locked host memory, which
+// saves the call a copy or two behind this launch.
+//
+// A warp takes a piece of an image row of up to kPieceVecs 16-byte words,
+// aligned in the destination: words whose bytes lie at the same alignment in
+// the canvas (16-byte aligned rows) are moved as they are, others are put
+// together from five 4-byte words by funnel shifts; the ends of the row go
+// byte by byte.  Bound by memory: 8192 x 8192 takes 28 us (134 MB, 4.7 TB/s;
+// pieces of 512 words, a whole row per warp, took 17 us more: too many rows
+// open at once).  128 images of 128..2048 pixels a side, 157 MB, 101 us;
+// a call with them 3.34 -> 3.13 ms, 3839 x 2161 0.163 -> 0.136 ms (every 4-byte
+// word, and every byte of an odd row, used to be gathered by itself).
+constexpr int kPieceVecs = 128;
+
+__host__ __device__ inline int row_pieces(int cols) {
+    return cols < 16 * kPieceVecs ? 1 : (cols / 16 + kPieceVecs - 1) / kPieceVecs;
 }
 
-// Batched copy-out: grid (per-image CTAs, images); image blockIdx.y, whose
-// `user` pointer is the caller's dense image (row r at user + r * cols), or
-// null for an image staged by the host.
-
-// Canvas `cur` -> dense image: one aligned 4-byte word of the destination
-// per thread, gathered from the canvas; the partial words at the two ends of
-// the image are written byte by byte.
-__global__ void copy_out_batch_kernel(const Ctrl* __restrict__ c, const uint8_t* __restrict__ a0,
-                                      const uint8_t* __restrict__ a1, const uint8_t* __restrict__ a2,
-                                      const ImgDesc* __restrict__ imgs) {
-    const ImgDesc d = imgs[blockIdx.y];
-    if (!d.user) return;
-    const unsigned cur = __ldcg(&c->cur);
-    const uint8_t* canvas = (cur == 0 ? a0 : (cur == 1 ? a1 : a2)) + d.off + (long long)kPadY * d.pitch + kPadX;
-    const uintptr_t ad = reinterpret_cast<uintptr_t>(d.user);
-    const int m = (int)(ad & 3u);
-    uint32_t* dw = reinterpret_cast<uint32_t*>(ad - (uintptr_t)m);
-    const long long nbytes = (long long)d.rows * d.cols;
-    const long long total = (m + nbytes + 3) / 4;
-    for (long long w = blockIdx.x * (long long)blockDim.x + threadIdx.x; w < total;
-         w += (long long)gridDim.x * blockDim.x) {
-        const long long l0 = 4 * w - m;  // image byte index of the word's first byte
-        long long first = l0 < 0 ? 0 : l0;
-        long long r = first / d.cols;
-        int col = (int)(first - r * d.cols);
-        uint32_t v = 0;
-        int nb = 0;
-        for (int b = (int)(first - l0); b < 4 && l0 + b < nbytes; ++b) {
-            v |= (uint32_t)canvas[r * d.pitch + col] << (8 * b);
-            ++nb;
-            if (++col == d.cols) {
-                col = 0;
-                ++r;
+__device__ __forceinline__ void copy_rows(const uint8_t* __restrict__ canvas, long long pitch,
+                                          uint8_t* __restrict__ user, int rows, int cols, int warp, int nwarps,
+                                          int lane) {
+    const int pieces = row_pieces(cols);
+    const int total = rows * pieces;
+    for (int t = warp; t < total; t += nwarps) {
+        const int r = pieces == 1 ? t : t / pieces, pc = t - r * pieces;
+        const uint8_t* src = canvas + r * pitch;
+        uint8_t* dst = user + (long long)r * cols;
+        const int head = min(cols, (int)(-reinterpret_cast<uintptr_t>(dst) & 15u));
+        const int nvec = (cols - head) / 16;
+        const int v1 = min(nvec, (pc + 1) * kPieceVecs);
+        uint4* dv = reinterpret_cast<uint4*>(dst + head);
+        if (head == 0) {
+#pragma unroll 4
+            for (int v = pc * kPieceVecs + lane; v < v1; v += 32) dv[v] = reinterpret_cast<const uint4*>(src)[v];
+        } else {
+            const uint32_t* sw = reinterpret_cast<const uint32_t*>(src + (head & ~3));
+            const uint32_t sh = (uint32_t)(head & 3) * 8u;
+#pragma unroll 4
+            for (int v = pc * kPieceVecs + lane; v < v1; v += 32) {
+                const uint32_t* q = sw + 4 * v;
+                const uint32_t w0 = q[0], w1 = q[1], w2 = q[2], w3 = q[3], w4 = q[4];
+                dv[v] = make_uint4(__funnelshift_r(w0, w1, sh), __funnelshift_r(w1, w2, sh),
+                                   __funnelshift_r(w2, w3, sh), __funnelshift_r(w3, w4, sh));
             }
         }
-        if (nb == 4) {
-            dw[w] = v;
-        } else {
-            uint8_t* db = reinterpret_cast<uint8_t*>(dw + w);
-            for (int b = 0; b < 4; ++b)
-                if (l0 + b >= 0 && l0 + b < nbytes) db[b] = (uint8_t)(v >> (8 * b));
+        if (pc == pieces - 1) {
+            if (lane < head) dst[lane] = src[lane];
+            const int e = head + 16 * nvec + lane;
+            if (e < cols && lane < 16) dst[e] = src[e];
         }
     }
+}
+
+__global__ void __launch_bounds__(256) call_finish_kernel(FinishArgs a) {
+    const Ctrl* c = a.ctrl;
+    const int lane = threadIdx.x & 31, warp = (blockIdx.x * 256 + threadIdx.x) >> 5, nwarps = gridDim.x * 8;
+    const uint8_t* canvas = a.arena[__ldcg(&c->cur)];
+    if (a.imgs) {
+        const ImgDesc d = load_desc(a.imgs, blockIdx.y);
+        if (d.user && a.write)
+            copy_rows(canvas + d.off + (long long)kPadY * d.pitch + kPadX, d.pitch, d.user, d.rows, d.cols, warp, nwarps,
+                      lane);
+    } else if (a.write) {
+        copy_rows(canvas + (long long)kPadY * a.pitch + kPadX, a.pitch, a.user, a.rows, a.cols, warp, nwarps, lane);
+    }
+    if (blockIdx.x == 0 && blockIdx.y == 0 && a.host_ctrl) {
+        const unsigned* cw = reinterpret_cast<const unsigned*>(c);
+        unsigned* hw = reinterpret_cast<unsigned*>(a.host_ctrl);
+        for (int i = threadIdx.x; i < (int)(sizeof(Ctrl) / 4); i += 256) hw[i] = __ldcg(cw + i);
+        if (a.host_img_k)
+            for (int i = threadIdx.x; i < a.nimg; i += 256) a.host_img_k[i] = __ldcg(a.img_k + i);
+    }
+}
+
+cudaError_t launch_call_finish(const FinishArgs& a, int sms, cudaStream_t s) {
+    // One image: up to eight CTAs per SM.  A batch: the CTAs of its largest
+    // image, limited to sixteen per SM over all images.
+    long long gx = 1;
+    if (a.write) gx = ((long long)a.rows * row_pieces(a.cols) + 7) / 8;
+    const unsigned gy = a.imgs ? (unsigned)a.nimg : 1u;
+    const long long cap = a.imgs ? std::max(((long long)sms * 16 + gy - 1) / gy, 16ll) : (long long)sms * 8;
+    gx = std::min(std::max(gx, 1ll), cap);
+    call_finish_kernel<<<dim3((unsigned)gx, gy), 256, 0, s>>>(a);
+    return cudaGetLastError();
 }
 
 // tile_img[b] = the image that fused tile b belongs to.
@@ -227,23 +242,6 @@ __global__ void tile_map_kernel(const ImgDesc* __restrict__ imgs, int nimg, int 
     const int t0 = imgs[i].tile0;
     const int t1 = i + 1 < nimg ? imgs[i + 1].tile0 : total_tiles;
     for (int t = t0 + threadIdx.x; t < t1; t += blockDim.x) tile_img[t] = i;
-}
-
-static unsigned batch_copy_ctas(long long max_words, int nimg, int sms) {
-    long long g = (max_words + 2047) / 2048;
-    const long long cap = nimg > 0 ? ((long long)sms * 16 + nimg - 1) / nimg : 1;
-    const long long lim = cap > 16 ? cap : 16;
-    if (g > lim) g = lim;
-    if (g < 1) g = 1;
-    return (unsigned)g;
-}
-
-cudaError_t launch_copy_out_batch(const Ctrl* c, uint8_t* const arena[3], const ImgDesc* imgs, int nimg,
-                                  long long max_words, int sms, cudaStream_t s) {
-    if (nimg <= 0) return cudaSuccess;
-    copy_out_batch_kernel<<<dim3(batch_copy_ctas(max_words, nimg, sms), (unsigned)nimg), 256, 0, s>>>(
-        c, arena[0], arena[1], arena[2], imgs);
-    return cudaGetLastError();
 }
 
 __global__ void rms_kernel(const int* __restrict__ sum, const int* __restrict__ flag, int* __restrict__ out, int n) {

@@ -637,7 +637,7 @@ int run_hybrid(hgrms_ctx* h, const BatchImg* im, int n, int alpha, int beta, int
     const bool per_image_k = n > 1;
     // Layout: image i's canvas at offset off_i of each arena, its bitmap at
     // word bm_off_i of each bitmap arena, its tiles from tile0_i.
-    long long canvas_total = 0, bm_total = 0, tiles_total = 0, px_total = 0, max_words = 0;
+    long long canvas_total = 0, bm_total = 0, tiles_total = 0, px_total = 0;
     int max_rows = 1, max_cols = 1;
     int rc = ensure_table(h, (size_t)n, 0, false);
     if (rc < 0) return rc;
@@ -662,8 +662,6 @@ int run_hybrid(hgrms_ctx* h, const BatchImg* im, int n, int alpha, int beta, int
         bm_total += (long long)rows * d.bm_words;
         tiles_total += (long long)tiles_x * tiles_y;
         px_total += (long long)rows * cols;
-        const long long words = ((long long)rows * cols + 3) / 4 + 1;
-        if (words > max_words) max_words = words;
         if (rows > max_rows) max_rows = rows;
         if (cols > max_cols) max_cols = cols;
     }
@@ -776,10 +774,9 @@ int run_hybrid(hgrms_ctx* h, const BatchImg* im, int n, int alpha, int beta, int
                                         im[i].ptr, (size_t)d.cols, (size_t)d.cols, (size_t)d.rows,
                                         cudaMemcpyHostToDevice, s));
         }
-        HG_TRY(h, hg::launch_ctrl_init(h->ctrl, (unsigned)max_k, s));
-        HG_TRY(h, cudaMemsetAsync(h->bitmaps, 0, 4 * (size_t)bm_total * sizeof(uint32_t), s));
-        HG_TRY(h, cudaMemsetAsync(h->bar, 0, sizeof(hg::GridBar), s));
-        if (per_image_k) HG_TRY(h, cudaMemsetAsync(h->img_k, 0, (h->img_k_cap + (size_t)n) * sizeof(unsigned), s));
+        // The four bitmaps are bm_total 16-byte words.
+        HG_TRY(h, hg::launch_call_init(h->ctrl, (unsigned)max_k, h->bitmaps, bm_total, h->bar, h->img_k,
+                                       per_image_k ? (long long)h->img_k_cap + n : 0, h->sms, s));
         for (int i = 0; i < launches; ++i) {
             if (timed) HG_TRY(h, record(h->events[2 * i]));
             if (i < fused_launches) {
@@ -803,17 +800,22 @@ int run_hybrid(hgrms_ctx* h, const BatchImg* im, int n, int alpha, int beta, int
             }
             if (timed) HG_TRY(h, record(h->events[2 * i + 1]));
         }
-        if (!write_back || max_k == 0) {
-            // a trial, or no pass ran (the images are unchanged): no copy-out
-        } else if (n == 1 && im[0].dev) {
-            HG_TRY(h, hg::launch_copy_out(h->ctrl, h->canvas, h->host_desc[0].pitch, im[0].ptr, im[0].rows, im[0].cols,
-                                          h->sms, s));
-        } else {
-            HG_TRY(h, hg::launch_copy_out_batch(h->ctrl, h->canvas, h->d_desc, n, max_words, h->sms, s));
-        }
-        HG_TRY(h, cudaMemcpyAsync(h->host_ctrl, h->ctrl, sizeof(hg::Ctrl), cudaMemcpyDeviceToHost, s));
-        if (per_image_k)
-            HG_TRY(h, cudaMemcpyAsync(h->host_img_k, h->img_k, (size_t)n * sizeof(unsigned), cudaMemcpyDeviceToHost, s));
+        // Images out (a trial leaves them as they are, and without a pass they
+        // are unchanged), k to the host.
+        hg::FinishArgs fa = {};
+        fa.ctrl = h->ctrl;
+        for (int c = 0; c < 3; ++c) fa.arena[c] = h->canvas[c];
+        fa.imgs = n > 1 ? h->d_desc : nullptr;
+        fa.nimg = n;
+        fa.user = im[0].ptr;
+        fa.pitch = h->host_desc[0].pitch;
+        fa.rows = max_rows;
+        fa.cols = max_cols;
+        fa.write = write_back && max_k > 0 && (n > 1 || im[0].dev);
+        fa.host_ctrl = h->host_ctrl;
+        fa.img_k = h->img_k;
+        fa.host_img_k = per_image_k ? h->host_img_k : nullptr;
+        HG_TRY(h, hg::launch_call_finish(fa, h->sms, s));
         return HGRMS_OK;
     };
     if (ms) HG_TRY(h, cudaEventRecord(h->tune_ev[0], s));
@@ -824,7 +826,7 @@ int run_hybrid(hgrms_ctx* h, const BatchImg* im, int n, int alpha, int beta, int
         std::vector<uint8_t> key(sizeof(a) + 16 * sizeof(long long));
         memcpy(key.data(), &a, sizeof(a));
         const long long extra[16] = {beta, T, fused_launches, list_loop, launches, write_back, max_k, n,
-                                     (long long)(uintptr_t)im[0].ptr, im[0].rows, im[0].cols, max_words,
+                                     (long long)(uintptr_t)im[0].ptr, im[0].rows, im[0].cols, 0,
                                      timed, bm_total, (long long)(uintptr_t)h->host_ctrl,
                                      (long long)(uintptr_t)h->host_img_k};
         memcpy(key.data() + sizeof(a), extra, sizeof(extra));
@@ -1035,7 +1037,7 @@ int denoise_one(hgrms_ctx* h, uint8_t* img, int rows, int cols, int alpha, int b
         HG_TRY(h, cudaMemcpy2DAsync(ca + hg::kPadY * p.pitch + hg::kPadX, (size_t)p.pitch, img,
                                     (size_t)cols, (size_t)cols, (size_t)rows, cudaMemcpyHostToDevice, s));
     }
-    HG_TRY(h, hg::launch_ctrl_init(h->ctrl, (unsigned)max_k, s));
+    HG_TRY(h, hg::launch_call_init(h->ctrl, (unsigned)max_k, nullptr, 0, nullptr, nullptr, 0, h->sms, s));
     // Map 0 is written by the first launch; the launches clear the others.
     if (p.map_words > 0) HG_TRY(h, cudaMemsetAsync(h->chg_maps, 0, map_bytes, s));
     // The change bitmaps start empty; each list pass clears one for a later pass.
@@ -1092,7 +1094,19 @@ int denoise_one(hgrms_ctx* h, uint8_t* img, int rows, int cols, int alpha, int b
             HG_TRY(h, hg::launch_plain(beta, a, s));
         if (timed) HG_TRY(h, cudaEventRecord(h->events[2 * i + 1], s));
     }
-    if (dev) HG_TRY(h, hg::launch_copy_out(h->ctrl, h->canvas, p.pitch, img, rows, cols, h->sms, s));
+    if (dev || sync_and_finish) {
+        hg::FinishArgs fa = {};
+        fa.ctrl = h->ctrl;
+        for (int c = 0; c < 3; ++c) fa.arena[c] = h->canvas[c];
+        fa.nimg = 1;
+        fa.user = img;
+        fa.pitch = p.pitch;
+        fa.rows = rows;
+        fa.cols = cols;
+        fa.write = dev;
+        fa.host_ctrl = sync_and_finish ? h->host_ctrl : nullptr;
+        HG_TRY(h, hg::launch_call_finish(fa, h->sms, s));
+    }
     h->stats.launches += p.launches;
     h->stats.passes_per_launch = p.T;
     h->stats.tile_rows = p.fused ? p.fe->TH : 0;
@@ -1100,7 +1114,6 @@ int denoise_one(hgrms_ctx* h, uint8_t* img, int rows, int cols, int alpha, int b
     h->stats.ctas_per_launch = p.fused ? (long long)p.tiles_x * p.tiles_y
                                        : (long long)((cols + 31) / 32) * ((rows + 7) / 8);
     if (!sync_and_finish) return HGRMS_OK;
-    HG_TRY(h, cudaMemcpyAsync(h->host_ctrl, h->ctrl, sizeof(hg::Ctrl), cudaMemcpyDeviceToHost, s));
     HG_TRY(h, cudaStreamSynchronize(s));
     const hg::Ctrl c = *h->host_ctrl;
     if (!dev) {
