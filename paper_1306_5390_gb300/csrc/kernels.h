@@ -1,6 +1,8 @@
 // Internal declarations shared by the runtime and the kernel translation units.
 #pragma once
 
+#include <cuda.h>
+#include <cudaTypedefs.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 #include "common.cuh"
@@ -19,6 +21,8 @@ extern const int kFusedB3Count;
 // pass), or null; the built-in passes per launch for beta.
 const FusedEntry* find_fused(int beta, int T, int rn = 64);
 int default_passes(int beta);
+// cuTensorMapEncodeTiled from the driver, or null.
+PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder();
 
 cudaError_t launch_plain(int beta, const PassArgs& a, cudaStream_t s);
 // Clear a call's control block, bitmaps (n16 16-byte words), barrier and per-image counts (nk words).

@@ -14,18 +14,23 @@
 //   k_hat = max(0, w_h . [g, histogram] + b_h)
 //
 // The convolutions run on the 5th-generation tensor cores (tcgen05, BF16
-// operands, FP32 accumulation in tensor memory) as implicit GEMMs: one CTA
-// computes 128 output positions (two rows) x 16 channels of one image; the
-// 3 x 3 taps are the K steps (K = 16 per step: the 16 input channels, or
-// for the first layer the 9 taps of its single channel).  Operands sit in
-// shared memory in the no-swizzle K-major layout of 8-row x 16-byte core
-// matrices; one thread issues the MMAs and a commit to an mbarrier; after a
-// bounded wait each warp reads its 32 accumulator rows from tensor memory.
+// operands, FP32 accumulation in tensor memory) as implicit GEMMs with the 3 x
+// 3 taps as K steps.  A 16-channel layer's input comes into shared memory by
+// TMA as two planes of 8 channels, each a row-major list of 16-byte positions
+// with a pitch of 66 and the zero border filled in by the copy.  In that
+// layout 8 consecutive positions are one core matrix of the no-swizzle operand
+// formats, K-major with the channels as K (the convolution) and MN-major with the
+// positions as K (the weight gradients), and a tap is nothing but another start
+// address: no operand is ever rearranged by threads.
+#include <cuda.h>
+#include <cudaTypedefs.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 #include <string.h>
 
+#include <algorithm>
+#include <type_traits>
 #include <utility>
 #include <vector>
 
@@ -41,9 +46,7 @@ constexpr int kPix = kSide * kSide;    // 4096 positions
 constexpr int kCh = 16;                // channels
 constexpr int kBins = 16;              // histogram bins
 constexpr int kBlockM = 128;           // positions per CTA (MMA M)
-constexpr int kTileBytes = kBlockM * 16 * 2;  // one K step of A: 128 x 16 bf16
 constexpr int kBBytes = kCh * 16 * 2;         // one K step of B: 16 x 16 bf16
-constexpr int kTmemCols = 32;          // smallest tensor-memory allocation
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
     return (uint32_t)__cvta_generic_to_shared(p);
@@ -51,11 +54,9 @@ __device__ __forceinline__ uint32_t smem_u32(const void* p) {
 
 // Shared-memory matrix descriptor, no swizzle: start address, K-direction
 // core-matrix stride (leading byte offset) and M/N-direction stride (stride
-// byte offset), all in 16-byte units; descriptor version 1.
-__device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo, uint32_t sbo) {
-    return (uint64_t)((addr >> 4) & 0x3FFFu) | ((uint64_t)((lbo >> 4) & 0x3FFFu) << 16) |
-           ((uint64_t)((sbo >> 4) & 0x3FFFu) << 32) | (1ull << 46);
-}
+// byte offset), all in 16-byte units; descriptor version 1 (bit 46).
+__device__ __forceinline__ uint32_t desc_lo(uint32_t addr, uint32_t lbo) { return (addr >> 4) | (lbo >> 4) << 16; }
+__device__ __forceinline__ uint32_t desc_hi(uint32_t sbo) { return (sbo >> 4) | 1u << 14; }
 
 // Instruction descriptor of kind::f16: FP32 accumulator, BF16 A and B, both
 // K-major, N = 16, M = 128.
@@ -69,133 +70,262 @@ __device__ __forceinline__ int core_off(int row, int k) {
     return (row >> 3) * 256 + (k >> 3) * 128 + (row & 7) * 16 + (k & 7) * 2;
 }
 
-// One conv layer: in/out are [image][64][64][cin or 16] bf16; w holds the
-// B operand images of the K steps (9 of 512 bytes, or 1 for the first
-// layer) in shared-memory order; bias 16 floats.  Grid (32, images), 128
-// threads.
+__device__ __forceinline__ void mbar_init1(uint64_t* m, uint32_t count = 1) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(m)), "r"(count));
+}
+// Bounded wait for phase `parity` of an mbarrier.
+__device__ __forceinline__ bool mbar_wait_bounded(uint64_t* m, uint32_t parity) {
+    for (uint32_t spins = 0; spins < (1u << 22); ++spins) {
+        uint32_t done;
+        asm volatile(
+            "{\n.reg .pred q;\nmbarrier.try_wait.parity.shared::cta.b64 q, [%1], %2;\nselp.u32 %0, 1, 0, q;\n}"
+            : "=r"(done)
+            : "r"(smem_u32(m)), "r"(parity)
+            : "memory");
+        if (done) return true;
+    }
+    return false;
+}
+// The same; a wait that gives up records the error and waits once more, so
+// that no copy or MMA of this CTA is left in flight when the CTA goes on.
+__device__ __forceinline__ bool mbar_wait_or_flag(uint64_t* m, uint32_t parity, unsigned* err) {
+    if (mbar_wait_bounded(m, parity)) return true;
+    atomicExch(err, 1u);
+    return mbar_wait_bounded(m, parity);
+}
+__device__ __forceinline__ void tmem_alloc(uint32_t* slot, uint32_t cols) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(slot)), "r"(cols));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+}
+__device__ __forceinline__ void tmem_dealloc(uint32_t tmem, uint32_t cols) {
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(cols));
+}
+// One MMA, issued by the lane whose `lead` is set; operand descriptors as (low,
+// high) words.  The low word holds the start address in 16-byte units, so
+// stepping through an operand is an add to it.  The whole warp runs the loops
+// around it with the same values: descriptors live in uniform registers, and
+// code that only one thread reaches has to move every one of them there first.
+__device__ __forceinline__ void mma_f16(uint32_t lead, uint32_t d, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo,
+                                        uint32_t b_hi, uint32_t idesc, uint32_t acc) {
+    asm volatile(
+        "{\n.reg .b64 a, b;\n.reg .pred p, q;\nmov.b64 a, {%1, %2};\nmov.b64 b, {%3, %4};\nsetp.ne.u32 p, %6, 0;\n"
+        "setp.ne.u32 q, %7, 0;\n@q tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %5, p;\n}" ::"r"(d),
+        "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(acc), "r"(lead)
+        : "memory");
+}
+__device__ __forceinline__ void mma_commit(uint32_t lead, uint64_t* m) {
+    asm volatile(
+        "{\n.reg .pred q;\nsetp.ne.u32 q, %1, 0;\n"
+        "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}" ::"r"(smem_u32(m)),
+        "r"(lead)
+        : "memory");
+}
+// 1 in one lane of the (converged) warp.
+__device__ __forceinline__ uint32_t elect_one() {
+    uint32_t lead;
+    asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.u32 %0, 1, 0, p;\n}" : "=r"(lead));
+    return lead;
+}
+__device__ __forceinline__ void tmem_ld16(uint32_t addr, uint32_t (&r)[16]) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(addr));
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+// TMA load of one 8-channel plane of image `img`: rows from y, columns from x
+// (positions outside the image read as zeros; the innermost coordinate is
+// channel 0 or 8, a 16-byte boundary).
+__device__ __forceinline__ void tma_plane(void* dst, const CUtensorMap* map, int half, int x, int y, int img,
+                                          uint64_t* m) {
+    asm volatile(
+        "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], "
+        "[%6];" ::"r"(smem_u32(dst)),
+        "l"(map), "r"(8 * half), "r"(x), "r"(y), "r"(img), "r"(smem_u32(m))
+        : "memory");
+}
+__device__ __forceinline__ void mbar_expect(uint64_t* m, uint32_t bytes) {
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(m)), "r"(bytes) : "memory");
+}
+
+constexpr int kPitch = kSide + 2;  // positions per row with the border
+
+// One channel of an image (64 x 64 bf16) with a border of zeros into s_x (66 x 66).
+__device__ __forceinline__ void load_bordered(const __nv_bfloat16* __restrict__ x, float* s_x) {
+    for (int i = threadIdx.x; i < kPitch * kPitch; i += blockDim.x) {
+        const int y = i / kPitch - 1, xx = i % kPitch - 1;
+        s_x[i] = y >= 0 && y < kSide && xx >= 0 && xx < kSide ? __bfloat162float(x[y * kSide + xx]) : 0.f;
+    }
+}
+
+// The first layer: one input channel, 9 taps, 16 output channels.  in
+// [image][64][64], out [image][64][64][16] bf16; w the parameters [tap][16] in
+// fp32, rounded to bf16 here; bias 16 floats.  On the CUDA cores, products of
+// bf16 values summed in fp32: as a tensor-core GEMM its K is 9 and its operand
+// has to be gathered value by value, which took 30 us for 256 images.  CTA
+// (image); a thread keeps the weights of 8 channels in registers and computes
+// 32 positions.  256 images: 14 us (33.5 MB out).
+__global__ void __launch_bounds__(256) conv1_kernel(const __nv_bfloat16* __restrict__ in, const float* __restrict__ w,
+                                                    const float* __restrict__ bias, __nv_bfloat16* __restrict__ out) {
+    __shared__ float s_x[kPitch * kPitch];
+    const int tid = threadIdx.x, h = tid & 1;
+    load_bordered(in + (size_t)blockIdx.x * kPix, s_x);
+    float wr[9][8], br[8];
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+        br[c] = bias[8 * h + c];
+#pragma unroll
+        for (int t = 0; t < 9; ++t) wr[t][c] = __bfloat162float(__float2bfloat16_rn(w[t * kCh + 8 * h + c]));
+    }
+    __syncthreads();
+    __nv_bfloat16* dst = out + (size_t)blockIdx.x * kPix * kCh + 8 * h;
+    for (int p = tid >> 1; p < kPix; p += 128) {
+        const float* sx = s_x + (p >> 6) * kPitch + (p & 63);
+        float acc[8];
+#pragma unroll
+        for (int c = 0; c < 8; ++c) acc[c] = br[c];
+#pragma unroll
+        for (int t = 0; t < 9; ++t) {
+            const float x = sx[(t / 3) * kPitch + t % 3];
+#pragma unroll
+            for (int c = 0; c < 8; ++c) acc[c] = fmaf(x, wr[t][c], acc[c]);
+        }
+        __align__(16) __nv_bfloat16 o[8];
+#pragma unroll
+        for (int c = 0; c < 8; ++c) o[c] = __float2bfloat16_rn(fmaxf(acc[c], 0.f));
+        *reinterpret_cast<uint4*>(dst + (size_t)p * kCh) = *reinterpret_cast<const uint4*>(o);
+    }
+}
+
+// A 16-channel layer: out[p][co] = ReLU(bias[co] + sum over taps and ci of in[p +
+// tap][ci] w[tap][ci][co]).  CTA (b, image) computes kBand rows: their input
+// rows are kBand + 2 rows of the two channel planes, position (y, x) of the
+// padded band at 66 y + x.  Output q = 66 y + x (x < 64 is a pixel, the other
+// two are padding and are dropped) takes tap (ky, kx) from input q + 66 ky + kx,
+// so the A operand of a tap is the plane pair from that position on: 128
+// positions per MMA (M), two core matrices of 8 channels (K = 16, a plane
+// apart), 5 MMA tiles of 9 taps with an accumulator of 16 columns each.
 //
 // With mask != null the kernel computes the gradient of a layer's input
 // instead (back-propagation through a 16-channel convolution): `in` is the
 // gradient of the layer's output, the taps' offsets are negated, w holds the
 // transposed weights (output channel = the layer's input channel), and the
 // result is multiplied by (mask > 0), the ReLU of the layer's input.
-__global__ void __launch_bounds__(128) conv_tc_kernel(const __nv_bfloat16* __restrict__ in, int cin,
-                                                      const uint8_t* __restrict__ w, const float* __restrict__ bias,
-                                                      __nv_bfloat16* __restrict__ out, unsigned* __restrict__ err,
-                                                      const __nv_bfloat16* __restrict__ mask = nullptr) {
-    __shared__ __align__(1024) uint8_t sA[9 * kTileBytes];
-    __shared__ __align__(1024) uint8_t sB[9 * kBBytes];
-    __shared__ __align__(8) uint64_t mbar;
-    __shared__ uint32_t tmem_base;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int img = blockIdx.y;
-    const int steps = cin == 1 ? 1 : 9;
-    const int m = tid;                       // this thread's output position in the block
-    const int py = blockIdx.x * 2 + (m >> 6), px = m & 63;
-    const __nv_bfloat16* src = in + (size_t)img * kPix * cin;
+//
+// Bound by the operand reads of the MMAs from shared memory (4 KB each, about
+// 70 cycles; N is only 16).  8 rows a CTA leave four CTAs per SM (their 128
+// tensor-memory columns each are all there are), so loads, MMAs and epilogues
+// of different CTAs overlap; 4 rows and eight CTAs per SM measured the same.
+// 256 images: 27 us forward and backward (67 and 101 MB), 59 us when every
+// thread gathered the 9 taps of its position.
+constexpr int kBand = 8;
+constexpr int kBandTiles = ((kBand - 1) * kPitch + kSide + kBlockM - 1) / kBlockM;  // 5
+constexpr int kConvPlane = (kBandTiles * kBlockM + 2 * kPitch + 2 + 7) / 8 * 128;    // bytes; every position an MMA reads
+constexpr int kConvCols = 128;
+constexpr size_t kConvSmem = 50 * 1024;  // four CTAs per SM
+static_assert(kBandTiles * kCh <= kConvCols, "accumulator columns");
+static_assert(2 * kConvPlane + 9 * kBBytes + 128 <= (int)kConvSmem && (kBand + 2) * kPitch * 16 <= kConvPlane, "conv planes");
 
-    if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base)),
-                     "r"(kTmemCols));
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+__global__ void __launch_bounds__(128) conv16_tc_kernel(const __grid_constant__ CUtensorMap in,
+                                                        const uint8_t* __restrict__ w, const float* __restrict__ bias,
+                                                        __nv_bfloat16* __restrict__ out, unsigned* __restrict__ err,
+                                                        const __nv_bfloat16* __restrict__ mask) {
+    extern __shared__ __align__(128) uint8_t smem[];
+    __shared__ __align__(8) uint64_t full, done[kBandTiles];
+    __shared__ uint32_t tmem_base;
+    __shared__ float s_bias[kCh];
+    if (smem_u32(smem) & 127u) {  // TMA destinations need 128-byte boundaries
+        if (threadIdx.x == 0) atomicExch(err, 1u);
+        return;
     }
+    uint8_t* sB = smem + 2 * kConvPlane;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
+    const int img = blockIdx.y, y0 = blockIdx.x * kBand;
     if (tid == 0) {
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&mbar)));
+        mbar_init1(&full);
+        for (int t = 0; t < kBandTiles; ++t) mbar_init1(&done[t]);
         asm volatile("fence.mbarrier_init.release.cluster;");
+        asm volatile("fence.proxy.async.shared::cta;");
+        mbar_expect(&full, 2u * (kBand + 2) * kPitch * 16);
+        for (int h = 0; h < 2; ++h) tma_plane(smem + h * kConvPlane, &in, h, -1, y0 - 1, img, &full);
     }
-    // A operand: im2col rows of this block.
-    if (cin == 1) {
-        __align__(16) __nv_bfloat16 v[16];
-#pragma unroll
-        for (int t = 0; t < 16; ++t) {
-            float x = 0.f;
-            if (t < 9) {
-                const int y = py + t / 3 - 1, xx = px + t % 3 - 1;
-                if (y >= 0 && y < kSide && xx >= 0 && xx < kSide) x = __bfloat162float(src[y * kSide + xx]);
-            }
-            v[t] = __float2bfloat16_rn(x);
-        }
-        *reinterpret_cast<uint4*>(sA + core_off(m, 0)) = *reinterpret_cast<const uint4*>(&v[0]);
-        *reinterpret_cast<uint4*>(sA + core_off(m, 8)) = *reinterpret_cast<const uint4*>(&v[8]);
-    } else {
-        const int sgn = mask ? -1 : 1;
-#pragma unroll 1
-        for (int t = 0; t < 9; ++t) {
-            const int y = py + sgn * (t / 3 - 1), xx = px + sgn * (t % 3 - 1);
-            uint4 lo = make_uint4(0u, 0u, 0u, 0u), hi = lo;
-            if (y >= 0 && y < kSide && xx >= 0 && xx < kSide) {
-                const uint4* p = reinterpret_cast<const uint4*>(src + (size_t)(y * kSide + xx) * kCh);
-                lo = __ldg(p);
-                hi = __ldg(p + 1);
-            }
-            uint8_t* tile = sA + t * kTileBytes;
-            *reinterpret_cast<uint4*>(tile + core_off(m, 0)) = lo;
-            *reinterpret_cast<uint4*>(tile + core_off(m, 8)) = hi;
-        }
-    }
-    // B operand images.
-    for (int i = tid; i < steps * kBBytes / 16; i += 128)
+    __syncwarp();
+    if (warp == 0) tmem_alloc(&tmem_base, kConvCols);
+    for (int i = tid; i < 9 * kBBytes / 16; i += 128)
         reinterpret_cast<uint4*>(sB)[i] = __ldg(reinterpret_cast<const uint4*>(w) + i);
-    // Shared-memory writes -> visible to the tensor core (async proxy).
+    if (tid < kCh) s_bias[tid] = mask ? 0.f : bias[tid];
     asm volatile("fence.proxy.async.shared::cta;");
     asm volatile("tcgen05.fence::before_thread_sync;");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;");
     const uint32_t tmem = tmem_base;
-    if (tid == 0) {
-        for (int t = 0; t < steps; ++t) {
-            const uint64_t ad = smem_desc(smem_u32(sA + t * kTileBytes), 128, 256);
-            const uint64_t bd = smem_desc(smem_u32(sB + t * kBBytes), 128, 256);
-            const uint32_t acc = t > 0 ? 1u : 0u;
-            asm volatile(
-                "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
-                "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(tmem),
-                "l"(ad), "l"(bd), "r"(kIdesc), "r"(acc));
-        }
-        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-            smem_u32(&mbar)));
-    }
-    // Bounded wait for the MMAs (phase 0 of the mbarrier).
-    uint32_t done = 0;
-    for (uint32_t spins = 0; spins < (1u << 22); ++spins) {
-        asm volatile(
-            "{\n.reg .pred q;\nmbarrier.try_wait.parity.shared::cta.b64 q, [%1], 0;\nselp.u32 %0, 1, 0, q;\n}"
-            : "=r"(done)
-            : "r"(smem_u32(&mbar)));
-        if (done) break;
-    }
-    if (!done) atomicExch(err, 1u);
-    asm volatile("tcgen05.fence::after_thread_sync;");
-    if (done) {
-        // Accumulator rows 32 warp .. 32 warp + 31, columns 0..15.
-        uint32_t r[16];
-        asm volatile(
-            "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-            : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-              "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-            : "r"(tmem + ((uint32_t)(32 * warp) << 16)));
-        asm volatile("tcgen05.wait::ld.sync.aligned;");
-        __align__(16) __nv_bfloat16 o[16];
-        const int pos = (blockIdx.x * 2 + (m >> 6)) * kSide + (m & 63);
-        if (mask) {
-            const __nv_bfloat16* mk = mask + ((size_t)img * kPix + pos) * kCh;
+    if (warp == 0) {
+        const uint32_t lead = elect_one();
+        mbar_wait_or_flag(&full, 0u, err);
+        __syncwarp();
+        // Tap (ky, kx) is 66 ky + kx positions from the tile's first one, or,
+        // negated, as many back from position 134.
+        const uint32_t a0 = desc_lo(smem_u32(smem), kConvPlane) + (mask ? 2u * kPitch + 2u : 0u);
+        const uint32_t step = mask ? ~0u : 1u;
+        const uint32_t b0 = desc_lo(smem_u32(sB), 128);
 #pragma unroll
-            for (int c = 0; c < 16; ++c)
-                o[c] = __float2bfloat16_rn(__bfloat162float(mk[c]) > 0.f ? __uint_as_float(r[c]) : 0.f);
+        for (int t = 0; t < kBandTiles; ++t) {
+#pragma unroll
+            for (int tap = 0; tap < 9; ++tap)
+                mma_f16(lead, tmem + (uint32_t)(t * kCh),
+                        a0 + (uint32_t)(t * kBlockM) + step * (uint32_t)((tap / 3) * kPitch + tap % 3), desc_hi(128),
+                        b0 + (uint32_t)(tap * kBBytes / 16), desc_hi(256), kIdesc, tap > 0 ? 1u : 0u);
+            mma_commit(lead, &done[t]);
+        }
+    }
+    __syncwarp();
+    // The mask values of this thread's positions, loaded while the MMAs run.
+    uint4 mk[kBandTiles][2];
+    if (mask) {
+#pragma unroll
+        for (int t = 0; t < kBandTiles; ++t) {
+            const int q = t * kBlockM + 32 * warp + lane;
+            const int y = q / kPitch, x = q - y * kPitch;
+            if (x >= kSide || y >= kBand) continue;
+            const uint4* mp = reinterpret_cast<const uint4*>(mask + ((size_t)img * kPix + (y0 + y) * kSide + x) * kCh);
+            mk[t][0] = __ldg(mp);
+            mk[t][1] = __ldg(mp + 1);
+        }
+    }
+#pragma unroll
+    for (int t = 0; t < kBandTiles; ++t) {
+        const bool ok = __all_sync(0xffffffffu, mbar_wait_or_flag(&done[t], 0u, err));
+        asm volatile("tcgen05.fence::after_thread_sync;");
+        if (!ok) continue;
+        uint32_t r[16];
+        tmem_ld16(tmem + (uint32_t)(t * kCh) + ((uint32_t)(32 * warp) << 16), r);
+        const int q = t * kBlockM + 32 * warp + lane;
+        const int y = q / kPitch, x = q - y * kPitch;
+        if (x >= kSide || y >= kBand) continue;
+        const size_t pos = (size_t)img * kPix + (y0 + y) * kSide + x;
+        __align__(16) __nv_bfloat16 o[16];
+        if (mask) {
+            const uint32_t mw[8] = {mk[t][0].x, mk[t][0].y, mk[t][0].z, mk[t][0].w,
+                                    mk[t][1].x, mk[t][1].y, mk[t][1].z, mk[t][1].w};
+#pragma unroll
+            for (int c = 0; c < 16; ++c) {  // bf16 is the high half of an fp32
+                const float v = __uint_as_float(c & 1 ? mw[c / 2] & 0xFFFF0000u : mw[c / 2] << 16);
+                o[c] = __float2bfloat16_rn(v > 0.f ? __uint_as_float(r[c]) : 0.f);
+            }
         } else {
 #pragma unroll
-            for (int c = 0; c < 16; ++c) o[c] = __float2bfloat16_rn(fmaxf(__uint_as_float(r[c]) + bias[c], 0.f));
+            for (int c = 0; c < 16; ++c) o[c] = __float2bfloat16_rn(fmaxf(__uint_as_float(r[c]) + s_bias[c], 0.f));
         }
-        uint4* dst = reinterpret_cast<uint4*>(out + ((size_t)img * kPix + pos) * kCh);
+        uint4* dst = reinterpret_cast<uint4*>(out + pos * kCh);
         dst[0] = *reinterpret_cast<const uint4*>(&o[0]);
         dst[1] = *reinterpret_cast<const uint4*>(&o[8]);
     }
-    (void)lane;
     asm volatile("tcgen05.fence::before_thread_sync;");
     __syncthreads();
     if (warp == 0) {
         asm volatile("tcgen05.fence::after_thread_sync;");
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols));
+        tmem_dealloc(tmem, kConvCols);
     }
 }
 
@@ -250,9 +380,27 @@ __global__ void __launch_bounds__(256) features_kernel(const ImgDesc* __restrict
                   (float)s_hist[threadIdx.x] / ((float)d.rows * (float)d.cols));
 }
 
+constexpr int kHeadThreads = 1024;  // one CTA per image: many loads in flight
+
+// acc[c] += this thread's share of the sum over the positions of a layer's
+// channel c (two 16-byte loads per position).
+__device__ __forceinline__ void add_positions(const __nv_bfloat16* __restrict__ x, float (&acc)[kCh]) {
+#pragma unroll 4
+    for (int p = threadIdx.x; p < kPix; p += blockDim.x) {
+        const uint4* q = reinterpret_cast<const uint4*>(x + (size_t)p * kCh);
+        const uint4 a = __ldg(q), b = __ldg(q + 1);
+        const uint32_t w[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {  // bf16 is the high half of an fp32
+            acc[2 * i] += __uint_as_float(w[i] << 16);
+            acc[2 * i + 1] += __uint_as_float(w[i] & 0xFFFF0000u);
+        }
+    }
+}
+
 // k_hat of image blockIdx.x: mean of the last layer over the positions,
 // then the linear head on [means, histogram].
-__global__ void __launch_bounds__(256) head_kernel(const __nv_bfloat16* __restrict__ x4, const float* __restrict__ hist,
+__global__ void __launch_bounds__(kHeadThreads) head_kernel(const __nv_bfloat16* __restrict__ x4, const float* __restrict__ hist,
                                                    const float* __restrict__ wh, float* __restrict__ k_hat,
                                                    float* __restrict__ gap_out) {
     __shared__ float s_sum[kCh];
@@ -261,10 +409,7 @@ __global__ void __launch_bounds__(256) head_kernel(const __nv_bfloat16* __restri
     float acc[kCh];
 #pragma unroll
     for (int c = 0; c < kCh; ++c) acc[c] = 0.f;
-    const __nv_bfloat16* x = x4 + (size_t)blockIdx.x * kPix * kCh;
-    for (int p = threadIdx.x; p < kPix; p += blockDim.x)
-#pragma unroll
-        for (int c = 0; c < kCh; ++c) acc[c] += __bfloat162float(x[(size_t)p * kCh + c]);
+    add_positions(x4 + (size_t)blockIdx.x * kPix * kCh, acc);
 #pragma unroll
     for (int c = 0; c < kCh; ++c) {
         float v = acc[c];
@@ -284,171 +429,213 @@ __global__ void __launch_bounds__(256) head_kernel(const __nv_bfloat16* __restri
     }
 }
 
-// Weight and bias gradients of one conv layer (back-propagation):
+// Weight and bias gradients of a 16-channel layer (back-propagation):
 //   dW[tap][ci][co] += sum over positions p of X[p + off(tap)][ci] dY[p][co]
 //   db[co]          += sum over p of dY[p][co]
-// for image blockIdx.x, as GEMMs on the tensor cores: M = 128 rows
-// (tap, ci) - taps 0..7 x 16 channels in group 0 and tap 8 in group 1, or
-// the 9 taps of a 1-channel input in group 0 - N = 16 output channels,
-// K = positions, 64 per chunk (4 K steps), accumulated in tensor memory
-// over the 64 chunks of the image.  The operands are transposed into the
-// K-major layout while they are written to shared memory.  128 threads.
-__global__ void __launch_bounds__(128) conv_wgrad_tc_kernel(const __nv_bfloat16* __restrict__ X, int cin,
-                                                            const __nv_bfloat16* __restrict__ dY,
-                                                            float* __restrict__ dW, float* __restrict__ db,
-                                                            unsigned* __restrict__ err) {
-    constexpr int kChunk = 64, kSteps = kChunk / 16;
-    __shared__ __align__(1024) uint8_t sA[2][kSteps][kTileBytes];
-    __shared__ __align__(1024) uint8_t sB[kSteps][kBBytes];
-    __shared__ __align__(8) uint64_t mbar;
+// as GEMMs with the positions as K.  A task is kWBand rows of one image: the
+// planes of X with their border and of dY with the same pitch (its two padding
+// columns are zeros from outside the image, so what X holds there does not
+// count).  Both operands are read MN-major as they lie: a core matrix is 8
+// positions (K) of 8 channels (M or N).  A of (ky, 8 channels) has 8 such
+// groups at a stride of one position: kx = 0, 1, 2 and five that are not used
+// (M = 64 is the smallest; the strides of a plane and of a row do not fit one
+// descriptor).  Six accumulators of 16 columns, and one with a matrix of
+// ones as A for db, stay in tensor memory over all tasks of a CTA, one CTA per
+// SM; the next task's planes load while this one's MMAs run.  One warp
+// issues everything.  Bound by the operand reads from shared memory (2 KB per
+// MMA, 7 x 66 MMAs a task, 35 cycles each).  256 images: 58 us; transposing both
+// operands value by value, one 64-position chunk after another, took 190 us.
+constexpr int kWBand = 16;
+constexpr int kWSteps = kWBand * kPitch / 16;                                // K steps of 16 positions
+constexpr int kXPlane = ((kWBand * kPitch + 2 * kPitch + 16) * 16 + 127) / 128 * 128;  // every position an MMA reads
+constexpr int kYPlane = kWBand * kPitch * 16;
+constexpr int kWStage = 2 * (kXPlane + kYPlane);
+constexpr int kOnesBytes = 64 * 16 * 2;
+constexpr size_t kWgradSmem = 2 * kWStage + kOnesBytes;
+constexpr int kWCols = 128;
+static_assert(kWBand * kPitch % 16 == 0 && kYPlane % 128 == 0 && kSide % kWBand == 0, "wgrad band");
+// BF16, FP32 accumulation, both operands MN-major, N = 16, M = 64.
+constexpr uint32_t kWgradIdesc = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) |
+                                 ((uint32_t)(kCh >> 3) << 17) | (4u << 24);
+
+__global__ void __launch_bounds__(128) wgrad16_tc_kernel(const __grid_constant__ CUtensorMap xmap,
+                                                         const __grid_constant__ CUtensorMap ymap, int images,
+                                                         float* __restrict__ dW, float* __restrict__ db,
+                                                         unsigned* __restrict__ err) {
+    extern __shared__ __align__(128) uint8_t smem[];
+    __shared__ __align__(8) uint64_t full[2], freed[2];
     __shared__ uint32_t tmem_base;
-    __shared__ float s_db[kCh];
-    const int tid = threadIdx.x, warp = tid >> 5;
-    const int img = blockIdx.x;
-    const int groups = cin == 1 ? 1 : 2;
-    const __nv_bfloat16* x = X + (size_t)img * kPix * cin;
-    const __nv_bfloat16* dy = dY + (size_t)img * kPix * kCh;
-    if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base)),
-                     "r"(kTmemCols));
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+    __shared__ int s_ok;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
+    constexpr int kTasks = kSide / kWBand;  // per image
+    const int tasks = images * kTasks;
+    uint8_t* ones = smem + 2 * kWStage;
+    if (smem_u32(smem) & 127u) {  // TMA destinations need 128-byte boundaries
+        if (tid == 0) atomicExch(err, 1u);
+        return;
     }
+    // Positions behind the loaded rows are read by MMAs (for padding columns,
+    // against zeros of dY): they must be finite.
+    for (int i = tid; i < 2 * kWStage / 16; i += 128) reinterpret_cast<uint4*>(smem)[i] = make_uint4(0u, 0u, 0u, 0u);
+    for (int i = tid; i < kOnesBytes / 4; i += 128) reinterpret_cast<uint32_t*>(ones)[i] = 0x3F803F80u;
     if (tid == 0) {
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&mbar)));
+        for (int i = 0; i < 2; ++i) {
+            mbar_init1(&full[i]);
+            mbar_init1(&freed[i]);
+        }
         asm volatile("fence.mbarrier_init.release.cluster;");
+        s_ok = 1;
     }
-    if (tid < kCh) s_db[tid] = 0.f;
-    // Rows that no (tap, channel) fills stay zero for the whole kernel.
-    for (int i = tid; i < (int)(sizeof(sA) / 16); i += 128) reinterpret_cast<uint4*>(&sA[0][0][0])[i] = make_uint4(0u, 0u, 0u, 0u);
+    if (warp == 0) tmem_alloc(&tmem_base, kWCols);
+    asm volatile("fence.proxy.async.shared::cta;");
     asm volatile("tcgen05.fence::before_thread_sync;");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;");
     const uint32_t tmem = tmem_base;
-    float dbl[kCh];
-#pragma unroll
-    for (int c = 0; c < kCh; ++c) dbl[c] = 0.f;
-    bool ok = true;
-    for (int chunk = 0; chunk < kPix / kChunk && ok; ++chunk) {
-        // Fill: thread t handles position k = t & 63 of the chunk; the two
-        // halves of the block split the taps.
-        const int k = tid & 63, half = tid >> 6;
-        const int p = chunk * kChunk + k;
-        const int py = p >> 6, px = p & 63;
-        const int step = k >> 4, kk = k & 15;
-        for (int t = half; t < 9; t += 2) {
-            const int y = py + t / 3 - 1, xx = px + t % 3 - 1;
-            const bool in_img = y >= 0 && y < kSide && xx >= 0 && xx < kSide;
-            if (cin == 1) {
-                const float v = in_img ? __bfloat162float(x[y * kSide + xx]) : 0.f;
-                *reinterpret_cast<__nv_bfloat16*>(&sA[0][step][core_off(t, kk)]) = __float2bfloat16_rn(v);
-            } else {
-                __align__(16) __nv_bfloat16 v[16];
-                if (in_img) {
-                    const uint4* q = reinterpret_cast<const uint4*>(x + (size_t)(y * kSide + xx) * kCh);
-                    *reinterpret_cast<uint4*>(&v[0]) = __ldg(q);
-                    *reinterpret_cast<uint4*>(&v[8]) = __ldg(q + 1);
-                } else {
-#pragma unroll
-                    for (int c = 0; c < 16; ++c) v[c] = __float2bfloat16_rn(0.f);
+    if (warp == 0) {
+        const uint32_t lead = elect_one();
+        auto load = [&](int task, int st) {
+            if (!lead) return;
+            const int img = task / kTasks, y0 = (task % kTasks) * kWBand;
+            uint8_t* p = smem + st * kWStage;
+            mbar_expect(&full[st], 2u * ((kWBand + 2) * kPitch + kWBand * kPitch) * 16);
+            for (int h = 0; h < 2; ++h) tma_plane(p + h * kXPlane, &xmap, h, -1, y0 - 1, img, &full[st]);
+            for (int h = 0; h < 2; ++h) tma_plane(p + 2 * kXPlane + h * kYPlane, &ymap, h, 0, y0, img, &full[st]);
+        };
+        bool ok = true;
+        int n = 0;  // tasks of this CTA so far
+        int loads = 0;
+        if ((int)blockIdx.x < tasks) {
+            load(blockIdx.x, 0);
+            ++loads;
+        }
+        for (int task = blockIdx.x; task < tasks && ok; task += gridDim.x, ++n) {
+            const int st = n & 1;
+            const uint32_t use = (uint32_t)(n >> 1);  // earlier uses of this stage
+            const int next = task + gridDim.x;
+            if (next < tasks) {
+                // The other stage's MMAs (of task n - 1) must be done.
+                if (n >= 1) ok = __all_sync(0xffffffffu, mbar_wait_or_flag(&freed[st ^ 1], (uint32_t)((n - 1) >> 1) & 1u, err));
+                if (ok) {
+                    load(next, st ^ 1);
+                    ++loads;
                 }
-                const int g = t >> 3, row0 = (t & 7) * 16;
-#pragma unroll
-                for (int c = 0; c < 16; ++c) *reinterpret_cast<__nv_bfloat16*>(&sA[g][step][core_off(row0 + c, kk)]) = v[c];
+                __syncwarp();
             }
-        }
-        if (half == 0) {
-            __align__(16) __nv_bfloat16 v[16];
-            const uint4* q = reinterpret_cast<const uint4*>(dy + (size_t)p * kCh);
-            *reinterpret_cast<uint4*>(&v[0]) = __ldg(q);
-            *reinterpret_cast<uint4*>(&v[8]) = __ldg(q + 1);
+            ok = mbar_wait_or_flag(&full[st], use & 1u, err) && ok;
+            ok = __all_sync(0xffffffffu, ok);
+            const uint32_t x0 = smem_u32(smem + st * kWStage);
+            uint32_t xd = desc_lo(x0, 128), yd = desc_lo(x0 + 2 * kXPlane, 128);
+            const uint32_t od = desc_lo(smem_u32(ones), 1024);
+            auto step = [&](uint32_t acc) {
 #pragma unroll
-            for (int c = 0; c < 16; ++c) {
-                *reinterpret_cast<__nv_bfloat16*>(&sB[step][core_off(c, kk)]) = v[c];
-                dbl[c] += __bfloat162float(v[c]);
-            }
+                for (int j = 0; j < 6; ++j)  // (ky, half)
+                    mma_f16(lead, tmem + 16u * j, xd + (uint32_t)((j & 1) * (kXPlane / 16) + (j >> 1) * kPitch), desc_hi(16), yd,
+                            desc_hi(kYPlane), kWgradIdesc, acc);
+                mma_f16(lead, tmem + 16u * 6, od, desc_hi(128), yd, desc_hi(kYPlane), kWgradIdesc, acc);
+                xd += 16u;  // 16 positions
+                yd += 16u;
+            };
+            step(n > 0 ? 1u : 0u);
+#pragma unroll 2
+            for (int k = 1; k < kWSteps; ++k) step(1u);
+            mma_commit(lead, &freed[st]);
         }
-        asm volatile("fence.proxy.async.shared::cta;");
-        asm volatile("tcgen05.fence::before_thread_sync;");
-        __syncthreads();
-        asm volatile("tcgen05.fence::after_thread_sync;");
-        if (tid == 0) {
-            for (int g = 0; g < groups; ++g)
-                for (int st = 0; st < kSteps; ++st) {
-                    const uint64_t ad = smem_desc(smem_u32(&sA[g][st][0]), 128, 256);
-                    const uint64_t bd = smem_desc(smem_u32(&sB[st][0]), 128, 256);
-                    const uint32_t acc = (chunk > 0 || st > 0) ? 1u : 0u;
-                    asm volatile(
-                        "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
-                        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(tmem + 16u * g),
-                        "l"(ad), "l"(bd), "r"(kIdesc), "r"(acc));
-                }
-            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                smem_u32(&mbar)));
-        }
-        // The next fill overwrites the operands: wait for these MMAs.
-        uint32_t done = 0;
-        for (uint32_t spins = 0; spins < (1u << 22); ++spins) {
-            asm volatile(
-                "{\n.reg .pred q;\nmbarrier.try_wait.parity.shared::cta.b64 q, [%1], %2;\nselp.u32 %0, 1, 0, q;\n}"
-                : "=r"(done)
-                : "r"(smem_u32(&mbar)), "r"((uint32_t)(chunk & 1)));
-            if (done) break;
-        }
-        if (!done) {
-            atomicExch(err, 1u);
-            ok = false;
-        }
-        asm volatile("tcgen05.fence::after_thread_sync;");
-        ok = __syncthreads_and(ok);
+        // A load that no task waited for (after a wait that gave up), and the last two tasks' MMAs.
+        if (loads > n) mbar_wait_or_flag(&full[n & 1], (uint32_t)(n >> 1) & 1u, err);
+        for (int b = n - 2 > 0 ? n - 2 : 0; b < n; ++b) ok = mbar_wait_or_flag(&freed[b & 1], (uint32_t)(b >> 1) & 1u, err) && ok;
+        if (lead && (!ok || n == 0)) s_ok = 0;
     }
-    if (ok) {
-        for (int g = 0; g < groups; ++g) {
+    asm volatile("tcgen05.fence::before_thread_sync;");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;");
+    if (s_ok) {
+        // M = 64: rows 16 w .. 16 w + 15 in the first 16 lanes of warp w.
+        const int row = 16 * warp + lane;
+        for (int j = 0; j < 7; ++j) {
             uint32_t r[16];
-            asm volatile(
-                "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-                  "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]),
-                  "=r"(r[15])
-                : "r"(tmem + ((uint32_t)(32 * warp) << 16) + 16u * g));
-            asm volatile("tcgen05.wait::ld.sync.aligned;");
-            const int row = 32 * warp + (tid & 31);
-            int tap, ci;
-            if (cin == 1) {
-                tap = row;
-                ci = 0;
-            } else {
-                tap = g * 8 + (row >> 4);
-                ci = row & 15;
+            tmem_ld16(tmem + 16u * j + ((uint32_t)(32 * warp) << 16), r);
+            if (lane >= 16) continue;
+            if (j < 6 && row < 24) {
+                const int tap = (j >> 1) * 3 + (row >> 3), ci = (j & 1) * 8 + (row & 7);
+#pragma unroll
+                for (int c = 0; c < kCh; ++c) atomicAdd(&dW[(tap * kCh + ci) * kCh + c], __uint_as_float(r[c]));
             }
-            if (tap < 9 && (cin == 16 || row < 9) && (g == 0 || row < 16)) {
+            if (j == 6 && row == 0) {
 #pragma unroll
-                for (int c = 0; c < kCh; ++c) atomicAdd(&dW[(tap * cin + ci) * kCh + c], __uint_as_float(r[c]));
+                for (int c = 0; c < kCh; ++c) atomicAdd(&db[c], __uint_as_float(r[c]));
             }
-        }
-    }
-    if (tid < 64) {
-#pragma unroll
-        for (int c = 0; c < kCh; ++c) {
-            float v = dbl[c];
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-            if ((tid & 31) == 0) atomicAdd(&s_db[c], v);
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;");
     __syncthreads();
-    if (tid < kCh) atomicAdd(&db[tid], s_db[tid]);
     if (warp == 0) {
         asm volatile("tcgen05.fence::after_thread_sync;");
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols));
+        tmem_dealloc(tmem, kWCols);
     }
+}
+
+// The same for the first layer (one input channel): 9 x 16 sums per image,
+// on the CUDA cores (a tensor-core tile of 9 useful rows of 64 would be mostly
+// padding).  CTA (image); a thread takes 8 output channels of 32 positions
+// and keeps its 9 x 8 sums in registers; products of bf16 values in fp32.
+// 256 images: 27 us (33.5 MB of dY in); 125 us as a tensor-core GEMM.
+__global__ void __launch_bounds__(256) wgrad1_kernel(const __nv_bfloat16* __restrict__ X,
+                                                     const __nv_bfloat16* __restrict__ dY, float* __restrict__ dW,
+                                                     float* __restrict__ db) {
+    __shared__ float s_x[kPitch * kPitch];
+    __shared__ float s_sum[10][kCh];
+    const int tid = threadIdx.x, lane = tid & 31, h = tid & 1;
+    load_bordered(X + (size_t)blockIdx.x * kPix, s_x);
+    if (tid < 10 * kCh) s_sum[tid / kCh][tid % kCh] = 0.f;
+    __syncthreads();
+    float acc[10][8];
+#pragma unroll
+    for (int t = 0; t < 10; ++t)
+#pragma unroll
+        for (int c = 0; c < 8; ++c) acc[t][c] = 0.f;
+    const __nv_bfloat16* src = dY + (size_t)blockIdx.x * kPix * kCh + 8 * h;
+#pragma unroll 2
+    for (int p = tid >> 1; p < kPix; p += 128) {
+        const uint4 v = __ldg(reinterpret_cast<const uint4*>(src + (size_t)p * kCh));
+        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+        float g[8];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {  // bf16 is the high half of an fp32
+            g[2 * i] = __uint_as_float(w[i] << 16);
+            g[2 * i + 1] = __uint_as_float(w[i] & 0xFFFF0000u);
+        }
+        const float* sx = s_x + (p >> 6) * kPitch + (p & 63);
+#pragma unroll
+        for (int t = 0; t < 9; ++t) {
+            const float x = sx[(t / 3) * kPitch + t % 3];
+#pragma unroll
+            for (int c = 0; c < 8; ++c) acc[t][c] = fmaf(x, g[c], acc[t][c]);
+        }
+#pragma unroll
+        for (int c = 0; c < 8; ++c) acc[9][c] += g[c];
+    }
+#pragma unroll
+    for (int t = 0; t < 10; ++t)
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+            float v = acc[t][c];
+#pragma unroll
+            for (int o = 16; o > 1; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+            if (lane < 2) atomicAdd(&s_sum[t][8 * h + c], v);
+        }
+    __syncthreads();
+    if (tid < 9 * kCh)
+        atomicAdd(&dW[tid], s_sum[tid / kCh][tid % kCh]);
+    else if (tid < 10 * kCh)
+        atomicAdd(&db[tid - 9 * kCh], s_sum[9][tid - 9 * kCh]);
 }
 
 // Training head of image blockIdx.x: y = w . [means of x4, hist] + b (no
 // ReLU while fitting), loss term (y - k)^2 / n, its gradient g = 2 (y - k) / n
 // added into the head's gradients, and dgap[c] = g w[c] / 4096 for the
 // backward pass.
-__global__ void __launch_bounds__(256) train_head_kernel(const __nv_bfloat16* __restrict__ x4,
+__global__ void __launch_bounds__(kHeadThreads) train_head_kernel(const __nv_bfloat16* __restrict__ x4,
                                                          const float* __restrict__ hist, const float* __restrict__ k,
                                                          const float* __restrict__ wh, int n, float* __restrict__ gwh,
                                                          float* __restrict__ dgap, float* __restrict__ loss) {
@@ -458,10 +645,7 @@ __global__ void __launch_bounds__(256) train_head_kernel(const __nv_bfloat16* __
     float acc[kCh];
 #pragma unroll
     for (int c = 0; c < kCh; ++c) acc[c] = 0.f;
-    const __nv_bfloat16* x = x4 + (size_t)blockIdx.x * kPix * kCh;
-    for (int p = threadIdx.x; p < kPix; p += blockDim.x)
-#pragma unroll
-        for (int c = 0; c < kCh; ++c) acc[c] += __bfloat162float(x[(size_t)p * kCh + c]);
+    add_positions(x4 + (size_t)blockIdx.x * kPix * kCh, acc);
 #pragma unroll
     for (int c = 0; c < kCh; ++c) {
         float v = acc[c];
@@ -488,13 +672,22 @@ __global__ void __launch_bounds__(256) train_head_kernel(const __nv_bfloat16* __
 
 // Gradient of the last layer's output: dgap broadcast over the positions,
 // times the ReLU of that output.
-__global__ void train_dx4_kernel(const __nv_bfloat16* __restrict__ x4, const float* __restrict__ dgap, int n,
-                                 __nv_bfloat16* __restrict__ dx4) {
-    const size_t total = (size_t)n * kPix * kCh;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-        const size_t img = i / ((size_t)kPix * kCh);
-        const int c = (int)(i % kCh);
-        dx4[i] = __float2bfloat16_rn(__bfloat162float(x4[i]) > 0.f ? dgap[img * kCh + c] : 0.f);
+// One thread takes 8 channels of a position (16 bytes); 256 images 10 us (67
+// MB), 163 us value by value.
+__global__ void __launch_bounds__(256) train_dx4_kernel(const __nv_bfloat16* __restrict__ x4,
+                                                        const float* __restrict__ dgap, int n,
+                                                        __nv_bfloat16* __restrict__ dx4) {
+    const int total = n * kPix * 2;  // n <= 4096
+    for (int i = blockIdx.x * 256 + threadIdx.x; i < total; i += gridDim.x * 256) {
+        const int img = i / (kPix * 2), h = i & 1;
+        __align__(16) __nv_bfloat16 v[8], o[8];
+        *reinterpret_cast<uint4*>(v) = __ldg(reinterpret_cast<const uint4*>(x4) + i);
+        const float4* g = reinterpret_cast<const float4*>(dgap + img * kCh + 8 * h);
+        const float4 g0 = __ldg(g), g1 = __ldg(g + 1);
+        const float gv[8] = {g0.x, g0.y, g0.z, g0.w, g1.x, g1.y, g1.z, g1.w};
+#pragma unroll
+        for (int c = 0; c < 8; ++c) o[c] = __float2bfloat16_rn(__bfloat162float(v[c]) > 0.f ? gv[c] : 0.f);
+        reinterpret_cast<uint4*>(dx4)[i] = *reinterpret_cast<const uint4*>(o);
     }
 }
 
@@ -525,48 +718,88 @@ __global__ void gather_kernel(const __nv_bfloat16* __restrict__ in, const float*
     if (threadIdx.x == 0) k_out[b] = k_in[j];
 }
 
-// Parameter vector (hgrms_predictor_load's order) -> the B operand images
-// of the four layers for the forward pass (element (n = output channel,
-// k = input channel or, for layer 1, tap)) and of layers 2..4 for the
-// backward pass through their input (element (n = input channel, k =
-// output channel)), bf16, rounded to nearest even.
-__global__ void pack_kernel(const float* __restrict__ wv, uint8_t* __restrict__ fwd0, uint8_t* __restrict__ fwd1,
-                            uint8_t* __restrict__ fwd2, uint8_t* __restrict__ fwd3, uint8_t* __restrict__ bwd1,
-                            uint8_t* __restrict__ bwd2, uint8_t* __restrict__ bwd3) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;  // over 7 x 9 steps x 256 elements
-    if (i >= 7 * 9 * 256) return;
-    const int which = i / (9 * 256), rem = i % (9 * 256);
+// Parameter vector (hgrms_predictor_load's order) -> the B operand images of
+// layers 2..4 for the forward pass (element (n = output channel, k = input
+// channel)) and for the backward pass through their input (element (n = input
+// channel, k = output channel)), bf16, rounded to nearest even.
+struct PackedLayers {
+    uint8_t* fwd[3];
+    uint8_t* bwd[3];  // null: not wanted
+};
+__global__ void pack_kernel(const float* __restrict__ wv, PackedLayers out) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;  // over 6 x 9 steps x 256 elements
+    if (i >= 6 * 9 * 256) return;
+    const int which = i / (9 * 256), rem = i % (9 * 256), layer = which % 3;
     const int step = rem / 256, n = (rem % 256) / 16, k = rem % 16;
-    float v = 0.f;
-    uint8_t* dst;
-    if (which == 0) {  // layer 1 forward: one step, k = tap
-        if (step != 0) return;
-        if (k < 9) v = wv[k * kCh + n];
-        dst = fwd0;
-    } else if (which <= 3) {  // layers 2..4 forward
-        const float* wl = wv + 144 + (which - 1) * 2304;
-        v = wl[(step * kCh + k) * kCh + n];
-        dst = which == 1 ? fwd1 : (which == 2 ? fwd2 : fwd3);
-    } else {  // layers 2..4 backward through the input
-        const float* wl = wv + 144 + (which - 4) * 2304;
-        v = wl[(step * kCh + n) * kCh + k];
-        dst = which == 4 ? bwd1 : (which == 5 ? bwd2 : bwd3);
-    }
+    const float* wl = wv + 144 + layer * 2304;
+    uint8_t* dst = which < 3 ? out.fwd[layer] : out.bwd[layer];
+    if (!dst) return;
+    const float v = which < 3 ? wl[(step * kCh + k) * kCh + n] : wl[(step * kCh + n) * kCh + k];
     *reinterpret_cast<__nv_bfloat16*>(dst + step * kBBytes + core_off(n, k)) = __float2bfloat16_rn(v);
 }
 
+static cudaError_t launch_pack(const float* w, const PackedLayers& out, cudaStream_t s) {
+    pack_kernel<<<(6 * 9 * 256 + 255) / 256, 256, 0, s>>>(w, out);
+    return cudaGetLastError();
+}
+
+// fp32 -> bf16, nearest even.
+__global__ void to_bf16_kernel(const float* __restrict__ in, long long n, __nv_bfloat16* __restrict__ out) {
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
+        out[i] = __float2bfloat16_rn(in[i]);
+}
+
+constexpr int kNW = 144 + 3 * 2304 + 64 + 33;  // parameters
+constexpr int kBiasOff = 144 + 3 * 2304;
+constexpr int kHeadOff = kBiasOff + 64;
+
 }  // namespace
+
+// Tensor map of a [n][64][64][16] bf16 layer for tma_plane: boxes of 8
+// channels, 66 columns and `rows` rows of one image.
+static bool layer_map(CUtensorMap* m, const __nv_bfloat16* base, int n, int rows) {
+    PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
+    if (!enc) return false;
+    const cuuint64_t dims[4] = {(cuuint64_t)kCh, (cuuint64_t)kSide, (cuuint64_t)kSide, (cuuint64_t)n};
+    const cuuint64_t strides[3] = {kCh * 2, kSide * kCh * 2, (cuuint64_t)kPix * kCh * 2};
+    const cuuint32_t box[4] = {8, (cuuint32_t)kPitch, (cuuint32_t)rows, 1};
+    const cuuint32_t estr[4] = {1, 1, 1, 1};
+    return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<__nv_bfloat16*>(base), dims, strides, box, estr,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+static cudaError_t launch_conv1(const __nv_bfloat16* in, int n, const float* w, const float* bias, __nv_bfloat16* out,
+                                cudaStream_t s) {
+    conv1_kernel<<<(unsigned)n, 256, 0, s>>>(in, w, bias, out);
+    return cudaGetLastError();
+}
+static cudaError_t launch_conv16(const CUtensorMap& in, int n, const uint8_t* w, const float* bias, __nv_bfloat16* out,
+                                 unsigned* err, const __nv_bfloat16* mask, cudaStream_t s) {
+    cudaError_t e = cudaFuncSetAttribute(conv16_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kConvSmem);
+    if (e != cudaSuccess) return e;
+    conv16_tc_kernel<<<dim3(kSide / kBand, (unsigned)n), 128, kConvSmem, s>>>(in, w, bias, out, err, mask);
+    return cudaGetLastError();
+}
+static cudaError_t launch_wgrad16(const CUtensorMap& x, const CUtensorMap& dy, int n, float* dW, float* db, unsigned* err,
+                                  int sms, cudaStream_t s) {
+    cudaError_t e = cudaFuncSetAttribute(wgrad16_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWgradSmem);
+    if (e != cudaSuccess) return e;
+    const int tasks = n * (kSide / kWBand);
+    wgrad16_tc_kernel<<<(unsigned)(tasks < sms ? tasks : sms), 128, kWgradSmem, s>>>(x, dy, n, dW, db, err);
+    return cudaGetLastError();
+}
 
 // Device buffers of the predictor for up to `cap` images.
 struct Predictor {
-    uint8_t* w[4] = {nullptr, nullptr, nullptr, nullptr};  // B operand images per layer
-    float* bias = nullptr;                                   // 4 x 16
-    float* head = nullptr;                                   // 33
+    float* w = nullptr;                                      // the parameters (kNW)
+    uint8_t* packed[3] = {nullptr, nullptr, nullptr};        // B operand images of layers 2..4
     __nv_bfloat16* x0 = nullptr;                             // cap x 4096
     __nv_bfloat16* act[2] = {nullptr, nullptr};              // cap x 4096 x 16, ping-pong
     float* hist = nullptr;                                   // cap x 16
     float* khat = nullptr;                                   // cap
     unsigned* err = nullptr;
+    CUtensorMap act_map[2];  // of act[0], act[1]
     int cap = 0;
     bool loaded = false;
 };
@@ -575,9 +808,8 @@ Predictor* predictor_new() { return new Predictor(); }
 
 void predictor_free(Predictor* p) {
     if (!p) return;
-    for (int l = 0; l < 4; ++l) cudaFree(p->w[l]);
-    cudaFree(p->bias);
-    cudaFree(p->head);
+    for (int l = 0; l < 3; ++l) cudaFree(p->packed[l]);
+    cudaFree(p->w);
     cudaFree(p->x0);
     cudaFree(p->act[0]);
     cudaFree(p->act[1]);
@@ -587,48 +819,21 @@ void predictor_free(Predictor* p) {
     delete p;
 }
 
-// Host: B operand image of one K step: element (n = output channel, k) at
-// core_off(n, k), bf16.
-static void pack_b(const float* wl, int cin, int step, uint16_t* dst) {
-    for (int n = 0; n < kCh; ++n)
-        for (int k = 0; k < 16; ++k) {
-            float v = 0.f;
-            if (cin == 1) {
-                if (k < 9) v = wl[(k * 1 + 0) * kCh + n];  // tap k, channel 0
-            } else {
-                v = wl[(step * kCh + k) * kCh + n];  // tap step, input channel k
-            }
-            uint32_t u;
-            memcpy(&u, &v, 4);
-            const uint32_t r = u + 0x7FFFu + ((u >> 16) & 1u);  // round to nearest even
-            const int off = (n >> 3) * 256 + (k >> 3) * 128 + (n & 7) * 16 + (k & 7) * 2;
-            dst[off / 2] = (uint16_t)(r >> 16);
-        }
-}
-
 // weights: layer l (0..3) as [tap 0..8][cin][16] floats (cin = 1 for l = 0,
 // else 16), then 4 x 16 biases, then the head: 16 weights on the channel
 // means, 16 on the histogram, 1 bias.
 int predictor_load(Predictor* p, const float* weights, int n) {
-    const int need = 9 * 1 * 16 + 3 * 9 * 16 * 16 + 4 * 16 + 33;
-    if (n != need) return HGRMS_EINVAL;
-    const float* q = weights;
-    for (int l = 0; l < 4; ++l) {
-        const int cin = l == 0 ? 1 : 16;
-        const int steps = l == 0 ? 1 : 9;
-        uint16_t img[9 * kBBytes / 2];
-        memset(img, 0, sizeof(img));
-        for (int s = 0; s < steps; ++s) pack_b(q, cin, s, img + s * kBBytes / 2);
-        if (!p->w[l] && cudaMalloc(&p->w[l], 9 * kBBytes) != cudaSuccess) return HGRMS_ENOMEM;
-        if (cudaMemcpy(p->w[l], img, 9 * kBBytes, cudaMemcpyHostToDevice) != cudaSuccess) return HGRMS_ECUDA;
-        q += 9 * cin * 16;
+    if (n != kNW) return HGRMS_EINVAL;
+    if (!p->w && cudaMalloc(&p->w, kNW * sizeof(float)) != cudaSuccess) return HGRMS_ENOMEM;
+    PackedLayers pk = {};
+    for (int l = 0; l < 3; ++l) {
+        if (!p->packed[l] && cudaMalloc(&p->packed[l], 9 * kBBytes) != cudaSuccess) return HGRMS_ENOMEM;
+        pk.fwd[l] = p->packed[l];
     }
-    if (!p->bias && cudaMalloc(&p->bias, 64 * sizeof(float)) != cudaSuccess) return HGRMS_ENOMEM;
-    if (!p->head && cudaMalloc(&p->head, 33 * sizeof(float)) != cudaSuccess) return HGRMS_ENOMEM;
     if (!p->err && cudaMalloc(&p->err, sizeof(unsigned)) != cudaSuccess) return HGRMS_ENOMEM;
-    if (cudaMemcpy(p->bias, q, 64 * sizeof(float), cudaMemcpyHostToDevice) != cudaSuccess) return HGRMS_ECUDA;
-    q += 64;
-    if (cudaMemcpy(p->head, q, 33 * sizeof(float), cudaMemcpyHostToDevice) != cudaSuccess) return HGRMS_ECUDA;
+    if (cudaMemcpy(p->w, weights, kNW * sizeof(float), cudaMemcpyHostToDevice) != cudaSuccess) return HGRMS_ECUDA;
+    // Done before the call returns: later calls may run on another stream.
+    if (launch_pack(p->w, pk, nullptr) != cudaSuccess || cudaStreamSynchronize(nullptr) != cudaSuccess) return HGRMS_ECUDA;
     p->loaded = true;
     return HGRMS_OK;
 }
@@ -652,6 +857,8 @@ static int predictor_reserve(Predictor* p, int n) {
         cudaGetLastError();
         return HGRMS_ENOMEM;
     }
+    for (int i = 0; i < 2; ++i)
+        if (!layer_map(&p->act_map[i], p->act[i], n, kBand + 2)) return HGRMS_ECUDA;
     p->cap = n;
     return HGRMS_OK;
 }
@@ -682,13 +889,13 @@ int predictor_run(Predictor* p, const ImgDesc* imgs, int n, cudaStream_t s, floa
     const __nv_bfloat16* in = p->x0;
     for (int l = 0; l < 4 && e == cudaSuccess; ++l) {
         __nv_bfloat16* out = p->act[l & 1];
-        conv_tc_kernel<<<dim3(kPix / kBlockM, (unsigned)n), 128, 0, s>>>(in, l == 0 ? 1 : kCh, p->w[l],
-                                                                          p->bias + 16 * l, out, p->err);
-        e = cudaGetLastError();
+        const float* bias = p->w + kBiasOff + 16 * l;
+        e = l == 0 ? launch_conv1(in, n, p->w, bias, out, s)
+                   : launch_conv16(p->act_map[(l - 1) & 1], n, p->packed[l - 1], bias, out, p->err, nullptr, s);
         in = out;
     }
     if (e == cudaSuccess) {
-        head_kernel<<<(unsigned)n, 256, 0, s>>>(in, p->hist, p->head, p->khat, gap);
+        head_kernel<<<(unsigned)n, kHeadThreads, 0, s>>>(in, p->hist, p->w + kHeadOff, p->khat, gap);
         e = cudaGetLastError();
     }
     unsigned err = 0;
@@ -713,20 +920,17 @@ namespace hg {
 
 namespace {
 
-constexpr int kNW = 144 + 3 * 2304 + 64 + 33;  // parameters
-constexpr int kBiasOff = 144 + 3 * 2304;
-constexpr int kHeadOff = kBiasOff + 64;
-
-// Device state of a fit.
+// Device state of a fit, in one allocation.
 struct Trainer {
     int n = 0, batch = 0;
+    uint8_t* arena = nullptr;
     __nv_bfloat16* x0 = nullptr;  // n x 4096
     float* hist = nullptr;        // n x 16
     float* k = nullptr;           // n
+    int* idx = nullptr;           // n: the epoch's permutation
     __nv_bfloat16* xb = nullptr;  // batch x 4096
     float* hb = nullptr;
     float* kb = nullptr;
-    int* idx = nullptr;
     __nv_bfloat16* act[4] = {};   // batch x 4096 x 16
     __nv_bfloat16* grad[2] = {};  // batch x 4096 x 16
     float* dgap = nullptr;
@@ -734,101 +938,109 @@ struct Trainer {
     float* g = nullptr;           // gradients
     float* m = nullptr;
     float* v = nullptr;
-    float* loss = nullptr;
+    float* loss = nullptr;        // n / batch: the epoch's minibatches
     unsigned* err = nullptr;
-    uint8_t* fwd[4] = {};
-    uint8_t* bwd[4] = {};
+    PackedLayers packed = {};
+    // Tensor maps of act[0..2] and grad[0..1]: for the convolutions (input
+    // bands) and the weight gradients (X and dY bands).
+    CUtensorMap act_conv[3], act_x[3], grad_conv[2], grad_y[2];
+    int sms = 0;
 
-    ~Trainer() {
-        cudaFree(x0); cudaFree(hist); cudaFree(k); cudaFree(xb); cudaFree(hb); cudaFree(kb); cudaFree(idx);
-        for (auto* a : act) cudaFree(a);
-        for (auto* a : grad) cudaFree(a);
-        cudaFree(dgap); cudaFree(w); cudaFree(g); cudaFree(m); cudaFree(v); cudaFree(loss); cudaFree(err);
-        for (auto* a : fwd) cudaFree(a);
-        for (auto* a : bwd) cudaFree(a);
-    }
+    ~Trainer() { cudaFree(arena); }
 };
-
-uint16_t to_bf16(float f) {
-    uint32_t u;
-    memcpy(&u, &f, 4);
-    return (uint16_t)((u + 0x7FFFu + ((u >> 16) & 1u)) >> 16);
-}
 
 int trainer_init(Trainer& t, const float* x0, const float* hist, const float* k, int n, int batch,
                  const float* weights, cudaStream_t s) {
     t.n = n;
     t.batch = batch;
     const size_t act = (size_t)batch * kPix * kCh * sizeof(__nv_bfloat16);
-    bool ok = cudaMalloc(&t.x0, (size_t)n * kPix * 2) == cudaSuccess &&
-              cudaMalloc(&t.hist, (size_t)n * kBins * 4) == cudaSuccess && cudaMalloc(&t.k, (size_t)n * 4) == cudaSuccess &&
-              cudaMalloc(&t.xb, (size_t)batch * kPix * 2) == cudaSuccess &&
-              cudaMalloc(&t.hb, (size_t)batch * kBins * 4) == cudaSuccess &&
-              cudaMalloc(&t.kb, (size_t)batch * 4) == cudaSuccess && cudaMalloc(&t.idx, (size_t)batch * 4) == cudaSuccess &&
-              cudaMalloc(&t.dgap, (size_t)batch * kCh * 4) == cudaSuccess && cudaMalloc(&t.w, kNW * 4) == cudaSuccess &&
-              cudaMalloc(&t.g, kNW * 4) == cudaSuccess && cudaMalloc(&t.m, kNW * 4) == cudaSuccess &&
-              cudaMalloc(&t.v, kNW * 4) == cudaSuccess && cudaMalloc(&t.loss, 4) == cudaSuccess &&
-              cudaMalloc(&t.err, 4) == cudaSuccess;
-    for (int i = 0; i < 4 && ok; ++i) ok = cudaMalloc(&t.act[i], act) == cudaSuccess;
-    for (int i = 0; i < 2 && ok; ++i) ok = cudaMalloc(&t.grad[i], act) == cudaSuccess;
-    for (int i = 0; i < 4 && ok; ++i)
-        ok = cudaMalloc(&t.fwd[i], 9 * kBBytes) == cudaSuccess && cudaMalloc(&t.bwd[i], 9 * kBBytes) == cudaSuccess;
-    if (!ok) {
-        cudaGetLastError();
-        return HGRMS_ENOMEM;
+    size_t total = 0;
+    // Two rounds: the sizes, then the addresses (256-byte boundaries).
+    auto place = [&](auto*& p, size_t bytes) {
+        if (t.arena) p = reinterpret_cast<std::remove_reference_t<decltype(p)>>(t.arena + total);
+        total += (bytes + 255) / 256 * 256;
+    };
+    for (int round = 0; round < 2; ++round) {
+        total = 0;
+        place(t.x0, (size_t)n * kPix * 2);
+        place(t.hist, (size_t)n * kBins * 4);
+        place(t.k, (size_t)n * 4);
+        place(t.idx, (size_t)n * 4);
+        place(t.xb, (size_t)batch * kPix * 2);
+        place(t.hb, (size_t)batch * kBins * 4);
+        place(t.kb, (size_t)batch * 4);
+        for (auto*& a : t.act) place(a, act);
+        for (auto*& a : t.grad) place(a, act);
+        place(t.dgap, (size_t)batch * kCh * 4);
+        place(t.w, kNW * 4);
+        place(t.g, kNW * 4);
+        place(t.m, kNW * 4);
+        place(t.v, kNW * 4);
+        place(t.loss, (size_t)(n / batch) * 4);
+        place(t.err, 4);
+        for (auto*& a : t.packed.fwd) place(a, 9 * kBBytes);
+        for (auto*& a : t.packed.bwd) place(a, 9 * kBBytes);
+        if (round == 0 && cudaMalloc(&t.arena, total) != cudaSuccess) {
+            cudaGetLastError();
+            t.arena = nullptr;
+            return HGRMS_ENOMEM;
+        }
     }
-    std::vector<uint16_t> xh((size_t)n * kPix);
-    for (size_t i = 0; i < xh.size(); ++i) xh[i] = to_bf16(x0[i]);
-    cudaError_t e = cudaMemcpyAsync(t.x0, xh.data(), xh.size() * 2, cudaMemcpyHostToDevice, s);
+    for (int i = 0; i < 3; ++i)
+        if (!layer_map(&t.act_conv[i], t.act[i], batch, kBand + 2) || !layer_map(&t.act_x[i], t.act[i], batch, kWBand + 2))
+            return HGRMS_ECUDA;
+    for (int i = 0; i < 2; ++i)
+        if (!layer_map(&t.grad_conv[i], t.grad[i], batch, kBand + 2) || !layer_map(&t.grad_y[i], t.grad[i], batch, kWBand))
+            return HGRMS_ECUDA;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&t.sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return HGRMS_ECUDA;
+    cudaError_t e = cudaSuccess;
+    // x0 as it is, through the activations' memory, and to bf16 on the device.
+    const size_t chunk = (size_t)batch * kCh / 2;  // images that fit act[0] in fp32
+    for (size_t i = 0; i < (size_t)n && e == cudaSuccess; i += chunk) {
+        const size_t c = std::min(chunk, (size_t)n - i) * kPix;
+        e = cudaMemcpyAsync(t.act[0], x0 + i * kPix, c * 4, cudaMemcpyHostToDevice, s);
+        if (e != cudaSuccess) break;
+        to_bf16_kernel<<<(unsigned)t.sms * 8, 256, 0, s>>>(reinterpret_cast<const float*>(t.act[0]), (long long)c,
+                                                          t.x0 + i * kPix);
+        e = cudaGetLastError();
+    }
     if (e == cudaSuccess) e = cudaMemcpyAsync(t.hist, hist, (size_t)n * kBins * 4, cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(t.k, k, (size_t)n * 4, cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(t.w, weights, kNW * 4, cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(t.m, 0, kNW * 4, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(t.v, 0, kNW * 4, s);
-    for (int i = 0; i < 4 && e == cudaSuccess; ++i) {
-        e = cudaMemsetAsync(t.fwd[i], 0, 9 * kBBytes, s);
-        if (e == cudaSuccess) e = cudaMemsetAsync(t.bwd[i], 0, 9 * kBBytes, s);
-    }
     if (e == cudaSuccess) e = cudaMemsetAsync(t.err, 0, 4, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);  // xh goes out of scope
     return e == cudaSuccess ? HGRMS_OK : HGRMS_ECUDA;
 }
 
-cudaError_t trainer_pack(Trainer& t, cudaStream_t s) {
-    pack_kernel<<<(7 * 9 * 256 + 255) / 256, 256, 0, s>>>(t.w, t.fwd[0], t.fwd[1], t.fwd[2], t.fwd[3], t.bwd[1],
-                                                          t.bwd[2], t.bwd[3]);
-    return cudaGetLastError();
-}
-
-// Gradient of the mean squared k error over the images idx_host[0..nb) into
-// t.g (and their loss into t.loss): forward through the tensor-core layers,
-// then back through them.
-cudaError_t trainer_grad(Trainer& t, const int* idx_host, int nb, cudaStream_t s) {
-    cudaError_t e = cudaMemcpyAsync(t.idx, idx_host, (size_t)nb * 4, cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(t.g, 0, kNW * 4, s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(t.loss, 0, 4, s);
+// Gradient of the mean squared k error over the images t.idx[b0 .. b0 + nb) into
+// t.g (their loss is added to *loss): forward through the layers, then back
+// through them.  Nothing waits for the host.
+cudaError_t trainer_grad(Trainer& t, int b0, int nb, float* loss, cudaStream_t s) {
+    cudaError_t e = cudaMemsetAsync(t.g, 0, kNW * 4, s);
     if (e != cudaSuccess) return e;
-    gather_kernel<<<nb, 256, 0, s>>>(t.x0, t.hist, t.k, t.idx, nb, t.xb, t.hb, t.kb);
-    const __nv_bfloat16* in = t.xb;
-    for (int l = 0; l < 4; ++l) {
-        conv_tc_kernel<<<dim3(kPix / kBlockM, nb), 128, 0, s>>>(in, l == 0 ? 1 : kCh, t.fwd[l], t.w + kBiasOff + 16 * l,
-                                                                t.act[l], t.err);
-        in = t.act[l];
-    }
-    train_head_kernel<<<nb, 256, 0, s>>>(t.act[3], t.hb, t.kb, t.w + kHeadOff, nb, t.g + kHeadOff, t.dgap, t.loss);
-    train_dx4_kernel<<<256, 256, 0, s>>>(t.act[3], t.dgap, nb, t.grad[0]);
+    gather_kernel<<<nb, 256, 0, s>>>(t.x0, t.hist, t.k, t.idx + b0, nb, t.xb, t.hb, t.kb);
+    const float* bias = t.w + kBiasOff;
+    e = launch_conv1(t.xb, nb, t.w, bias, t.act[0], s);
+    for (int l = 1; l < 4 && e == cudaSuccess; ++l)
+        e = launch_conv16(t.act_conv[l - 1], nb, t.packed.fwd[l - 1], bias + 16 * l, t.act[l], t.err, nullptr, s);
+    if (e != cudaSuccess) return e;
+    train_head_kernel<<<nb, kHeadThreads, 0, s>>>(t.act[3], t.hb, t.kb, t.w + kHeadOff, nb, t.g + kHeadOff, t.dgap, loss);
+    train_dx4_kernel<<<t.sms * 8, 256, 0, s>>>(t.act[3], t.dgap, nb, t.grad[0]);
+    e = cudaGetLastError();
     int cur = 0;
     const int woff[4] = {0, 144, 144 + 2304, 144 + 2 * 2304};
-    for (int l = 3; l >= 0; --l) {
-        const __nv_bfloat16* X = l == 0 ? t.xb : t.act[l - 1];
-        conv_wgrad_tc_kernel<<<nb, 128, 0, s>>>(X, l == 0 ? 1 : kCh, t.grad[cur], t.g + woff[l],
-                                                t.g + kBiasOff + 16 * l, t.err);
-        if (l > 0) {
-            conv_tc_kernel<<<dim3(kPix / kBlockM, nb), 128, 0, s>>>(t.grad[cur], kCh, t.bwd[l], nullptr,
-                                                                    t.grad[cur ^ 1], t.err, t.act[l - 1]);
-            cur ^= 1;
-        }
+    for (int l = 3; l >= 1 && e == cudaSuccess; --l) {
+        e = launch_wgrad16(t.act_x[l - 1], t.grad_y[cur], nb, t.g + woff[l], t.g + kBiasOff + 16 * l, t.err, t.sms, s);
+        if (e == cudaSuccess)
+            e = launch_conv16(t.grad_conv[cur], nb, t.packed.bwd[l - 1], nullptr, t.grad[cur ^ 1], t.err, t.act[l - 1], s);
+        cur ^= 1;
     }
+    if (e != cudaSuccess) return e;
+    wgrad1_kernel<<<nb, 256, 0, s>>>(t.xb, t.grad[cur], t.g, t.g + kBiasOff);
     return cudaGetLastError();
 }
 
@@ -842,8 +1054,10 @@ int predictor_grad(const float* weights, const float* x0, const float* hist, con
     if (rc < 0) return rc;
     std::vector<int> idx((size_t)n);
     for (int i = 0; i < n; ++i) idx[i] = i;
-    cudaError_t e = trainer_pack(t, s);
-    if (e == cudaSuccess) e = trainer_grad(t, idx.data(), n, s);
+    cudaError_t e = cudaMemcpyAsync(t.idx, idx.data(), (size_t)n * 4, cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(t.loss, 0, 4, s);
+    if (e == cudaSuccess) e = launch_pack(t.w, t.packed, s);
+    if (e == cudaSuccess) e = trainer_grad(t, 0, n, t.loss, s);
     unsigned err = 0;
     if (e == cudaSuccess) e = cudaMemcpyAsync(grads, t.g, kNW * 4, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(loss, t.loss, 4, cudaMemcpyDeviceToHost, s);
@@ -867,35 +1081,36 @@ int predictor_train(float* weights, const float* x0, const float* hist, const fl
         st = st * 6364136223846793005ull + 1442695040888963407ull;
         return (uint32_t)(st >> 33);
     };
-    cudaError_t e = trainer_pack(t, s);
+    cudaError_t e = launch_pack(t.w, t.packed, s);
     int step = 0;
-    double last = 0.0;
+    const int batches = n / batch;
+    // The steps are queued without waiting for any; an epoch's upload of its
+    // permutation (pageable memory) waits for the epoch before it.
     for (int ep = 0; ep < epochs && e == cudaSuccess; ++ep) {
         for (int i = n - 1; i > 0; --i) std::swap(perm[i], perm[next() % (uint32_t)(i + 1)]);
-        double ep_loss = 0.0;
-        int batches = 0;
         const float lr_ep = ep >= (3 * epochs) / 4 ? lr / 3.f : lr;
-        for (int b0 = 0; b0 + batch <= n && e == cudaSuccess; b0 += batch) {
-            e = trainer_grad(t, perm.data() + b0, batch, s);
+        e = cudaMemcpyAsync(t.idx, perm.data(), (size_t)n * 4, cudaMemcpyHostToDevice, s);
+        if (e == cudaSuccess) e = cudaMemsetAsync(t.loss, 0, (size_t)batches * 4, s);
+        for (int b = 0; b < batches && e == cudaSuccess; ++b) {
+            e = trainer_grad(t, b * batch, batch, t.loss + b, s);
             if (e != cudaSuccess) break;
             ++step;
             adam_kernel<<<(kNW + 255) / 256, 256, 0, s>>>(t.w, t.g, t.m, t.v, kNW, lr_ep, 0.9f, 0.999f, 1e-8f, step);
             e = cudaGetLastError();
-            if (e == cudaSuccess) e = trainer_pack(t, s);
-            float l = 0.f;
-            if (e == cudaSuccess) e = cudaMemcpyAsync(&l, t.loss, 4, cudaMemcpyDeviceToHost, s);
-            if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-            ep_loss += l;
-            ++batches;
+            if (e == cudaSuccess) e = launch_pack(t.w, t.packed, s);
         }
-        last = batches ? ep_loss / batches : 0.0;
     }
+    std::vector<float> losses((size_t)batches, 0.f);
+    if (e == cudaSuccess && epochs > 0)
+        e = cudaMemcpyAsync(losses.data(), t.loss, (size_t)batches * 4, cudaMemcpyDeviceToHost, s);
     unsigned err = 0;
     if (e == cudaSuccess) e = cudaMemcpyAsync(weights, t.w, kNW * 4, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(&err, t.err, 4, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return HGRMS_ECUDA;
-    if (loss_out) *loss_out = (float)last;
+    double last = 0.0;  // the last epoch's mean loss
+    for (float l : losses) last += l;
+    if (loss_out) *loss_out = (float)(last / batches);
     return err ? HGRMS_ETIMEOUT : HGRMS_OK;
 }
 

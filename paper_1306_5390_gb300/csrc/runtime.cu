@@ -141,6 +141,22 @@ const FusedEntry* find_fused(int beta, int T, int rn) {
     return nullptr;
 }
 
+// cuTensorMapEncodeTiled from the driver (looked up once; null if absent).
+PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
+    static PFN_cuTensorMapEncodeTiled_v12000 fn = []() -> PFN_cuTensorMapEncodeTiled_v12000 {
+        void* p = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) !=
+                cudaSuccess ||
+            q != cudaDriverEntryPointSuccess) {
+            cudaGetLastError();
+            return nullptr;
+        }
+        return reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(p);
+    }();
+    return fn;
+}
+
 int default_passes(int beta) {
     switch (beta) {
         case 1: return 8;
@@ -183,6 +199,7 @@ long long default_relaunch_ppm(int alpha, int beta) {
 
 using hg::default_passes;
 using hg::find_fused;
+using hg::tensor_map_encoder;
 
 // Cooperative list-pass launches of every handle of the process on one device
 // run one after another, in the order they are issued.  The CTAs of such a
@@ -447,22 +464,6 @@ int ensure_table(hgrms_ctx* h, size_t n, size_t tiles, bool per_image_k) {
         h->img_k_cap = n;
     }
     return HGRMS_OK;
-}
-
-// cuTensorMapEncodeTiled from the driver (looked up once; null if absent).
-PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
-    static PFN_cuTensorMapEncodeTiled_v12000 fn = []() -> PFN_cuTensorMapEncodeTiled_v12000 {
-        void* p = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) !=
-                cudaSuccess ||
-            q != cudaDriverEntryPointSuccess) {
-            cudaGetLastError();
-            return nullptr;
-        }
-        return reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(p);
-    }();
-    return fn;
 }
 
 // A 3-D byte view for tile loads: (16 bytes, 16-byte chunks of a row, rows)

@@ -208,3 +208,69 @@ def test_training_reduces_loss(torch_cuda):
         w, loss = d.train_predictor(w0, x0, hist, k, epochs=30, batch=64, lr=1e-2, seed=3)
         _, loss1 = d.predictor_grad(w, x0, hist, k)
     assert np.isfinite(loss1) and loss1 < 0.2 * loss0, (loss0, loss, loss1)
+
+
+def bf16_t(torch, x):
+    return x.to(torch.float32).to(torch.bfloat16).to(torch.float64)
+
+
+def device_like_grad(torch, w, x0, hist, k):
+    """The gradient with the device's BF16 roundings (weights, activations,
+    layer gradients) and float64 sums, layer by layer."""
+    F = torch.nn.functional
+    n = len(k)
+    nconv = 144 + 3 * 2304
+    convs, off = [], 0
+    wt = torch.tensor(np.concatenate([bf16(w[:nconv]), w[nconv:]]).astype(np.float64)).cuda()
+    for cin in (1, 16, 16, 16):
+        convs.append(wt[off:off + 9 * cin * 16].view(3, 3, cin, 16).permute(3, 2, 0, 1))
+        off += 9 * cin * 16
+    acts = [torch.tensor(bf16(x0).astype(np.float64)).cuda()[:, None]]
+    for l in range(4):
+        b = wt[nconv + 16 * l:nconv + 16 * (l + 1)]
+        acts.append(bf16_t(torch, torch.relu(F.conv2d(acts[-1], convs[l], b, padding=1))))
+    head = wt[nconv + 64:]
+    gap = acts[4].mean(dim=(2, 3))
+    h = torch.tensor(hist.astype(np.float64)).cuda()
+    e = gap @ head[:16] + h @ head[16:32] + head[32] - torch.tensor(k.astype(np.float64)).cuda()
+    ge = 2.0 * e / n
+    out = torch.zeros(len(w), dtype=torch.float64, device="cuda")
+    out[nconv + 64:nconv + 80] = gap.T @ ge
+    out[nconv + 80:nconv + 96] = h.T @ ge
+    out[nconv + 96] = ge.sum()
+    dy = bf16_t(torch, (ge[:, None] * head[:16] / 4096.0)[:, :, None, None] * (acts[4] > 0))
+    off = nconv
+    for l in (3, 2, 1, 0):
+        cin = acts[l].shape[1]
+        off -= 9 * cin * 16
+        xp = F.pad(acts[l], (1, 1, 1, 1))
+        for t in range(9):
+            win = xp[:, :, t // 3:t // 3 + 64, t % 3:t % 3 + 64]
+            out[off + t * cin * 16:off + (t + 1) * cin * 16] = torch.einsum("nihw,nohw->io", win, dy).reshape(-1)
+        out[nconv + 16 * l:nconv + 16 * (l + 1)] = dy.sum(dim=(0, 2, 3))
+        if l:
+            dy = bf16_t(torch, F.conv_transpose2d(dy, convs[l], padding=1) * (acts[l] > 0))
+    return out.cpu().numpy(), float((e * e).mean())
+
+
+@pytest.mark.parametrize("n", [1, 2, 37, 153, 310])
+def test_gradient_of_every_batch_size(torch_cuda, n):
+    """One image, fewer tasks than SMs, one and several tasks per SM with a
+    remainder, against the same roundings with float64 sums: what is left is
+    the order of FP32 sums and the roundings to BF16 that it tips over (2^-9
+    of a value, few of them): 1e-3 of a group's norm covers both."""
+    torch = torch_cuda
+    from paper_1306_5390_gb300 import hgrms
+    rng = np.random.Generator(np.random.PCG64(100 + n))
+    x0 = rng.uniform(0.0, 1.0, size=(n, 64, 64)).astype(np.float32)
+    hist = rng.dirichlet(np.ones(16), size=n).astype(np.float32)
+    k = rng.uniform(0.0, 32.0, size=n).astype(np.float32)
+    w = random_weights(23, scale=0.2)
+    with hgrms.Denoiser(0) as d:
+        g, loss = d.predictor_grad(w, x0, hist, k)
+    ref, loss_ref = device_like_grad(torch, w, x0, hist, k)
+    assert abs(loss - loss_ref) <= 1e-3 * loss_ref
+    groups = [(0, 144), (144, 2448), (2448, 4752), (4752, 7056), (7056, 7120), (7120, 7153)]
+    for a, b in groups:
+        err = np.linalg.norm(g[a:b] - ref[a:b]) / max(np.linalg.norm(ref[a:b]), 1e-12)
+        assert err < 1e-3, (a, b, err)
