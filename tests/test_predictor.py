@@ -91,6 +91,37 @@ def test_features_match_definition(torch_cuda):
         np.testing.assert_allclose(hist[i], rh, rtol=1e-6, atol=1e-7, err_msg=str(im.shape))
 
 
+@pytest.mark.parametrize("rows,cols", [(1, 70), (63, 64), (129, 65), (70, 127), (64, 128), (130, 129), (66, 1023),
+                                              (65, 1025), (300, 259), (16500, 64), (20000, 3), (40, 4100)])
+def test_features_at_the_ends_of_their_ranges(torch_cuda, rows, cols, offset=1):
+    """Widths around a warp's columns and a lane's four, rows past the 256 a
+    16-bit sum holds, constant images (one histogram bin, full counters), odd
+    addresses.  Sums are whole numbers; the division rounds once (1e-6)."""
+    torch = torch_cuda
+    from paper_1306_5390_gb300 import hgrms
+    rng = np.random.Generator(np.random.PCG64(rows + cols))
+    imgs = [rng.integers(0, 256, size=(rows, cols), dtype=np.uint8), np.full((rows, cols), 255, np.uint8)]
+    buf = torch.zeros(2 * rows * cols + 64, dtype=torch.uint8, device="cuda")
+    views = []
+    for i, im in enumerate(imgs):
+        o = offset + i * (rows * cols + 2)
+        views.append(buf[o:o + rows * cols].view(rows, cols))
+        views[-1].copy_(torch.from_numpy(im))
+    with hgrms.Denoiser(0) as d:
+        d.load_predictor(1, random_weights(1))
+        _, x0, hist, _ = d.predict_k(1, views, features=True)
+    for i, im in enumerate(imgs):
+        r = np.arange(64)
+        r0, c0 = r * rows // 64, r * cols // 64
+        r1, c1 = np.maximum(r0 + 1, (r + 1) * rows // 64), np.maximum(c0 + 1, (r + 1) * cols // 64)
+        s = np.zeros((rows + 1, cols + 1), dtype=np.int64)
+        s[1:, 1:] = im.astype(np.int64).cumsum(0).cumsum(1)
+        cell = s[r1][:, c1] - s[r0][:, c1] - s[r1][:, c0] + s[r0][:, c0]
+        rx = cell / ((r1 - r0)[:, None] * (c1 - c0)[None, :] * 255.0)
+        np.testing.assert_allclose(x0[i], rx, rtol=0, atol=1e-6)
+        np.testing.assert_allclose(hist[i], np.bincount((im >> 4).ravel(), minlength=16) / im.size, rtol=1e-5, atol=1e-7)
+
+
 @pytest.mark.parametrize("seed", [2, 3])
 def test_network_matches_numpy(torch_cuda, seed):
     torch = torch_cuda
