@@ -265,15 +265,21 @@ __device__ __forceinline__ void add_image(int* img_n, int d, unsigned img, int l
     if (d != 0 && sum != 0 && __ffs(peers) - 1 == lane) atomicAdd(img_n + img, sum);
 }
 
-// Solo passes: a list of n pixels is left to CTA 0 when n P <= kSoloEvals
-// (P = (2 beta + 1)^2).  A pass of a handful of pixels is all latency: across
-// the grid 5.6 us with 152 CTAs and 6.4 us with 304, of which the barrier, the
-// append counter's round trip and the bitmap lookups are most; in one CTA,
-// with the lists and the claims in shared memory, 1.25 us for 30 pixels of
-// beta 2 and 5.4 us at the limit (beta 1, 205 pixels, four rounds of the
-// CTA's threads).
+// Short lists.  A pass of a handful of pixels is all latency.  Lists whose
+// (listed pixel, window position) pairs fit the grid's threads take the direct
+// path, one round of loads and one evaluation per thread (beta 1 and 2; for
+// wider windows most of the pairs would load for nothing): 8192 x 8192, beta 1,
+// 3.8-5 us a pass where a thread with nine positions in turn took 6.3-7.3, of
+// which the barrier is about 2 us.  Lists of at most kSoloPixels pixels are
+// left to CTA 0 alone, with the lists and the claims in shared memory: 1.25 us
+// a pass for 30 pixels of beta 2, 2.4 us for 44, 5.4 us for 205 of beta 1 (four
+// rounds of the CTA's threads, where the grid is faster again).
 constexpr unsigned kDirectD = 6;
+constexpr int kDirectB = 2;
+constexpr int kDescCache = 128;
 constexpr int kSoloEvals = 2048;
+template <int B>
+constexpr unsigned kSoloPixels = B == 1 ? 112u : (unsigned)(kSoloEvals / ((2 * B + 1) * (2 * B + 1)));
 constexpr int kSoloHash = 2 * kSoloEvals;        // claim table, at most half full
 constexpr int kSoloPasses = 1024;                // then the other CTAs' waits end
 constexpr unsigned kSoloClear = 1u << 16;        // largest list whose bitmap CTA 0 clears
@@ -392,7 +398,7 @@ __device__ __forceinline__ void solo_passes(const PassArgs& a, const ImgDesc& on
         uint32_t* l = list;
         list = next;
         next = l;
-        if (n == 0u || st.k >= max_k || n * P > kSoloEvals || passes >= kSoloPasses) break;
+        if (n == 0u || st.k >= max_k || n > kSoloPixels<B> || passes >= kSoloPasses) break;
     }
     st.n_cur = n;
     st.n_last = 0u;
@@ -468,6 +474,12 @@ __global__ void __launch_bounds__(kListThreads, 2) list_loop_kernel(PassArgs a) 
     const long long gthreads = (long long)gridDim.x * blockDim.x;
     const long long gtid = (long long)blockIdx.x * blockDim.x + tid;
     const long long warp_base = (long long)blockIdx.x * blockDim.x + (tid & ~31);
+    // Tasks are dealt to the CTAs a warp at a time: neighbours on a list are
+    // mostly neighbours in the image, and a warp's loads then share cache
+    // lines (a load of 32 lanes in 32 lines takes 32 turns in L1).  64
+    // photographs, first pass of 195,000 listed pixels: 25 us, 40 us when every
+    // lane went to another CTA.
+    const long long first_task = ((long long)warp * gridDim.x + blockIdx.x) * 32 + lane;
     // The single image as a table entry (its offsets are 0).
     ImgDesc one;
     if constexpr (!kBatch) {
@@ -481,6 +493,17 @@ __global__ void __launch_bounds__(kListThreads, 2) list_loop_kernel(PassArgs a) 
         one.bm_words = a.bm_words;
         one.user = nullptr;
     }
+    // Batches: the first images' table entries in shared memory (every barrier
+    // empties L1, so a table read costs a pass one more trip to L2).
+    constexpr int kCached = kBatch && B <= 4 ? kDescCache : 0;
+    __shared__ ImgDesc s_desc[kCached > 0 ? kCached : 1];
+    if constexpr (kCached > 0) {
+        for (int i = tid; i < min(a.nimg, kCached); i += kListThreads) s_desc[i] = load_desc(a.imgs, (unsigned)i);
+    }
+    auto desc = [&](unsigned img) -> ImgDesc {
+        if constexpr (!kBatch) return one;
+        else return img < (unsigned)kCached ? s_desc[img] : load_desc(a.imgs, img);
+    };
     constexpr int kXb = 16, kYb = 16;
     const int xb = kBatch ? a.xb : kXb, yb = kBatch ? a.yb : kYb;
     StagedList sl{stage_all + warp * StagedList::kCap, 0, 0u};
@@ -497,7 +520,7 @@ __global__ void __launch_bounds__(kListThreads, 2) list_loop_kernel(PassArgs a) 
 
     while (true) {
         int dn = 0;  // this thread's share of the change of N
-        if (st.n_cur <= (unsigned)(kSoloEvals / P) && st.n_cur <= a.list_cap && st.n_last <= kSoloClear &&
+        if (st.n_cur <= kSoloPixels<B> && st.n_cur <= a.list_cap && st.n_last <= kSoloClear &&
             st.n_last <= a.list_cap) {
             if (blockIdx.x == 0) {
                 solo_passes<B, kBatch>(a, one, base, xb, yb, max_k, k0, st, stage_all, s_queue, s_solo_n, evals, dn);
@@ -558,13 +581,14 @@ __global__ void __launch_bounds__(kListThreads, 2) list_loop_kernel(PassArgs a) 
             ctrl->list_n[(st.t + base + 2) & 3] = 0u;
         }
         const unsigned n = st.n_cur, nclr = st.n_last;
-        // The first list entry this thread reads (beta 1: entry tid *
-        // gridDim.x + blockIdx.x; wider windows: the entry of that task),
-        // loaded before the bitmap clearing below so that the two loads overlap.
+        // A short list: one thread per (listed pixel, window position).
+        const bool direct = B <= kDirectB && (long long)n * P <= gthreads && n <= a.list_cap;
+        // The list entry of this thread's first task, loaded before the bitmap clearing below so that the two
+        // loads overlap.
         uint32_t pk_first = 0u;
         if (n <= a.list_cap) {
-            const long long i0 = (long long)tid * gridDim.x + blockIdx.x;
-            const long long per = B == 1 ? 1 : W;
+            const long long i0 = first_task;
+            const long long per = direct ? P : (B == 1 ? 1 : W);
             if (i0 < (long long)n * per) pk_first = __ldcg(prev + (unsigned)(i0 / per));
         }
         // Clear bitmap sc (written by pass t - 2, read by pass t - 1) for pass
@@ -577,23 +601,77 @@ __global__ void __launch_bounds__(kListThreads, 2) list_loop_kernel(PassArgs a) 
                     unsigned img;
                     int y, x;
                     unpack_entry(clr[i], xb, yb, img, y, x);
-                    const ImgDesc d = kBatch ? load_desc(a.imgs, img) : one;
+                    const ImgDesc d = desc(img);
                     bm_clr[d.bm_off + (long long)y * d.bm_words + (x >> 5)] = 0u;
                 }
             } else {
                 for (long long i = gtid; i < a.bm_total; i += gthreads) bm_clr[i] = 0u;
             }
         }
-        if (n <= a.list_cap && B == 1) {
+        if (B <= kDirectB && direct) {
+            // Task (listed pixel p, window position): decides ownership of q
+            // from the list's bits of q's window rows up to p's (as below),
+            // and evaluates it, all from one round of loads.
+            const unsigned i = (unsigned)first_task;
+            bool ch = false, now = false, before = false;
+            uint32_t v = 0;
+            unsigned img = 0;
+            if (i < n * (unsigned)P) {
+                const int o = (int)(i % (unsigned)P);
+                int py, px;
+                unpack_entry(pk_first, xb, yb, img, py, px);
+                const ImgDesc d = desc(img);
+                const int dy = o / W - B, qy = py + dy, qx = px + o % W - B;
+                if (qy >= B && qy < d.rows - B && qx >= B && qx < d.cols - B) {
+                    const uint32_t* bmp = bm_prev + d.bm_off;
+                    const uint8_t* in = in_arena + d.off + (long long)kPadY * d.pitch + kPadX;
+                    const long long off = (long long)qy * d.pitch + qx;
+                    uint8_t* out = out_arena + d.off + (long long)kPadY * d.pitch + kPadX + off;
+                    constexpr int NW = (W + 3) / 4;
+                    uint32_t win[W][NW];
+                    const int was = __ldcg(out);
+                    uint32_t ahead = 0u;  // listed pixels of q's window before p (bit j: column qx - B + j)
+#pragma unroll
+                    for (int r = 0; r < W; ++r) {
+                        load_row_bytes<W>(in + off + (long long)(r - B) * d.pitch - B, win[r]);
+                        const int gy = qy - B + r;
+                        if (gy <= py) {
+                            const uint32_t bits = row_bits(bmp + (size_t)gy * d.bm_words, d.bm_words, qx - B) & ((1u << W) - 1u);
+                            ahead |= gy < py ? bits : bits & ((1u << (px - qx + B)) - 1u);
+                        }
+                    }
+                    if (ahead == 0u) {
+                        ++evals;
+                        const int ip = (int)((win[B][B / 4] >> (8 * (B % 4))) & 0xffu);
+                        const int nv = eval_window<B>(win, a.alpha);
+                        v = pack_entry(img, qy, qx, xb, yb);
+                        if (nv != was) *out = (uint8_t)nv;
+                        if (nv != (make_c ? ip : was)) {
+                            ch = true;
+                            atomicOr(bm_next + d.bm_off + (size_t)qy * d.bm_words + (qx >> 5), 1u << (qx & 31));
+                        }
+                        now = nv != ip;
+                        before = ip != was;
+                    }
+                }
+            }
+            const int delta = (now ? add : 0) - (before ? sub : 0);
+            dn += delta;
+            if (kBatch && a.img_k) {
+                mark_image(s_imgbits, now, img, lane);
+                mark_image(s_imgbits0, before && !now, img, lane);
+                add_image(a.img_n, delta, img, lane);
+            }
+            staged_append(sl, next, nnext, a.list_cap, ch, v, lane);
+        } else if (n <= a.list_cap && B == 1) {
             // beta 1: one thread per listed pixel p.  It loads p's 5 x 5
             // neighbourhood, the 3 x 3 window of the output canvas and the
             // list's bits of the rows up to p's, and evaluates every pixel q
             // of p's 3 x 3 window that p owns (no listed pixel of q's window
-            // precedes p in raster order) from those registers.  Listed
-            // pixels are dealt to the CTAs in turn.
-            long long i = (long long)tid * gridDim.x + blockIdx.x;
+            // precedes p in raster order) from those registers.
+            long long i = first_task;
             uint32_t pk = pk_first;
-            for (long long c0 = 0; c0 + blockIdx.x < (long long)n; c0 += gthreads, i += gthreads) {
+            for (long long c0 = 0; c0 + 32ll * blockIdx.x < (long long)n; c0 += gthreads, i += gthreads) {
                 const long long inext = i + gthreads;
                 const uint32_t pk_next = inext < (long long)n ? __ldcg(prev + (unsigned)inext) : 0u;
                 uint32_t chm = 0u;  // bit (dy + 1) * 3 + dx + 1: q = p + (dy, dx) goes on the next list
@@ -603,7 +681,7 @@ __global__ void __launch_bounds__(kListThreads, 2) list_loop_kernel(PassArgs a) 
                 int py = 0, px = 0;
                 if (i < (long long)n) {
                     unpack_entry(pk, xb, yb, img, py, px);
-                    const ImgDesc d = kBatch ? load_desc(a.imgs, img) : one;
+                    const ImgDesc d = desc(img);
                     const uint32_t* bmp = bm_prev + d.bm_off;
                     const uint8_t* in = in_arena + d.off + (long long)kPadY * d.pitch + kPadX;
                     uint8_t* out = out_arena + d.off + (long long)kPadY * d.pitch + kPadX;
@@ -672,14 +750,11 @@ __global__ void __launch_bounds__(kListThreads, 2) list_loop_kernel(PassArgs a) 
             // Chunks of one task per thread: task (listed pixel p, window
             // row dy) finds the pixels q = p + (dy, dx) that p owns and
             // queues them in shared memory (phase A); the CTA then evaluates
-            // its queue with every thread (phase B).  Tasks are dealt to the
-            // CTAs in turn (task c0 + tid * gridDim.x + blockIdx.x of chunk
-            // c0), so every CTA gets an equal share even when there are fewer
-            // tasks than threads.
+            // its queue with every thread (phase B).
             const long long ntask = (long long)n * W;
-            long long i = (long long)tid * gridDim.x + blockIdx.x;
+            long long i = first_task;
             uint32_t pk = pk_first;  // later chunks' entries are loaded one chunk early
-            for (long long c0 = 0; c0 + blockIdx.x < ntask; c0 += gthreads, i += gthreads) {
+            for (long long c0 = 0; c0 + 32ll * blockIdx.x < ntask; c0 += gthreads, i += gthreads) {
                 const long long inext = i + gthreads;
                 const uint32_t pk_next = inext < ntask ? __ldcg(prev + (unsigned)(inext / W)) : 0u;
                 // Phase A.  Ownership: no listed pixel of q's window precedes
@@ -694,7 +769,7 @@ __global__ void __launch_bounds__(kListThreads, 2) list_loop_kernel(PassArgs a) 
                 if (i < ntask) {
                     const int dy = (int)(i % W) - B;
                     unpack_entry(pk, xb, yb, img, py, px);
-                    const ImgDesc d = kBatch ? load_desc(a.imgs, img) : one;
+                    const ImgDesc d = desc(img);
                     qy = py + dy;
                     if (qy >= B && qy < d.rows - B) {
                         const uint32_t* bmp = bm_prev + d.bm_off;
@@ -753,7 +828,7 @@ __global__ void __launch_bounds__(kListThreads, 2) list_loop_kernel(PassArgs a) 
                         int y, x;
                         v = s_queue[j];
                         unpack_entry(v, xb, yb, qimg, y, x);
-                        const ImgDesc d = kBatch ? load_desc(a.imgs, qimg) : one;
+                        const ImgDesc d = desc(qimg);
                         const uint8_t* in = in_arena + d.off + (long long)kPadY * d.pitch + kPadX;
                         constexpr int NW = (W + 3) / 4;
                         uint32_t win[W][NW];
