@@ -75,9 +75,12 @@ struct FusedGeo {
     // memory); wider windows need more registers per thread and use warps of
     // 8-row bands.
     static constexpr int RN = RN_;
-    static_assert(RN == 64 || RN == 128, "tile rows");
-    static constexpr int kMinBlocks = RN == 64 ? 2 : 1;  // resident CTAs per SM
-    static constexpr int kThreads = (B == 1 ? 512 : 256) * (RN / 64);
+    // 32-row tiles are for calls of few tiles: the warps of a 64-row tile
+    // share its rows between twice as many CTAs, each on an SM that would idle
+    // (256 x 256, beta 1: 32.7 -> 25.6 us).
+    static_assert(RN == 32 || RN == 64 || RN == 128, "tile rows");
+    static constexpr int kMinBlocks = RN == 128 ? 1 : 2;  // resident CTAs per SM
+    static constexpr int kThreads = (B == 1 ? 512 : 256) * (RN == 128 ? 2 : 1);
     static constexpr int kWarps = kThreads / 32;
     static constexpr int kRows = RN / kWarps;        // rows per warp band (dense passes)
     static constexpr int TW = 240;                   // core tile width (pixels)
@@ -98,7 +101,7 @@ struct FusedGeo {
     // single-stage count measured faster); the second half of a warp's
     // candidate buffer then holds its work list of unsettled pixel pairs (at
     // most 4 per lane and row of a kAppendRows-row group).
-    static constexpr bool kStaged = B == 3 && kRows == 8;
+    static constexpr bool kStaged = B == 3 && kRows <= 8;
     static constexpr int kCandCap = kAppendRows * 256;  // per-warp candidate list
     static constexpr int kCandLimit = kStaged ? kCandCap / 2 : kCandCap;
     // Changed pixels kept per pass: a list pass needs at most eval_max /
@@ -1337,7 +1340,7 @@ fused_kernel(PassArgs a) {
 // Host-side description of one compiled (beta, T, tile rows) instance.
 struct FusedEntry {
     int beta, T, TH, TW;
-    int RN;    // rows computed per pass (64, or 128 for the tall tiles of large images)
+    int RN;    // rows computed per pass (64; 128 for large calls, 32 for calls of few tiles)
     int SH;    // tile rows with the halo (the TMA box height)
     bool tma;  // the kernel stages tiles by TMA when given tensor maps
     size_t smem;

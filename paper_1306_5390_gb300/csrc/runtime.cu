@@ -190,6 +190,13 @@ constexpr int kDefaultRelaunches = 3;
 // 629 M-pixel uneven batch; smaller calls keep the 64-row tiles, whose larger
 // tile count spreads better over the SMs.
 constexpr long long kTallMinPixels = 32ll << 20;
+// Calls of at most 3/2 32-row tiles per SM take those: 256 x 256 (30 tiles, 12
+// of 64 rows) 25.6 us in the fused launch against 32.7, 321 x 481 25.6 against
+// 33.8 (beta 1) and 35.8 (beta 2), 800 x 1200 (beta 2, 200 tiles) 33.8 against
+// 35.8, beta 3 27.6 against 33.8.  From there on the larger halo costs more than
+// the idle SMs: 720 x 1280, beta 1, 240 tiles, 33.8 us both; 1080 x 1920, beta
+// 3, 336 tiles, 44 against 35.
+constexpr long long low_tiles_max(int sms) { return 3ll * sms / 2; }
 constexpr long long kRelaunchMinPixels = 4ll << 20;
 constexpr size_t kMaxGraphs = 8;  // captured graphs kept per handle (HGRMS_OPT_GRAPH)
 constexpr int kMaxRelaunches = 8;
@@ -619,22 +626,25 @@ int run_hybrid(hgrms_ctx* h, const BatchImg* im, int n, int alpha, int beta, int
     const int T = tu.T;
     // Large calls (one image or a batch) take the tall tiles when they are
     // compiled for (beta, T) and compute fewer rows with them: at this size
-    // every SM still gets many tiles.
+    // every SM still gets many tiles.  Calls of few tiles take the low ones.
     const hg::FusedEntry* fe = find_fused(beta, T);
     if (!fe) return HGRMS_EINVAL;
     {
         const hg::FusedEntry* tall = find_fused(beta, T, 128);
-        long long px_call = 0, rows64 = 0, rows128 = 0;
-        for (int i = 0; i < n && tall; ++i) {
+        const hg::FusedEntry* low = find_fused(beta, T, 32);
+        long long px_call = 0, rows64 = 0, rows128 = 0, tiles32 = 0;
+        for (int i = 0; i < n && (tall || low); ++i) {
             const long long tx = (im[i].cols + fe->TW - 1) / fe->TW;
             px_call += (long long)im[i].rows * im[i].cols;
             rows64 += tx * ((im[i].rows + fe->TH - 1) / fe->TH) * 64;
-            rows128 += tx * ((im[i].rows + tall->TH - 1) / tall->TH) * 128;
+            if (tall) rows128 += tx * ((im[i].rows + tall->TH - 1) / tall->TH) * 128;
+            if (low) tiles32 += tx * ((im[i].rows + low->TH - 1) / low->TH);
         }
         if (tall && px_call >= kTallMinPixels && rows128 < rows64) fe = tall;
+        else if (low && tiles32 <= low_tiles_max(h->sms)) fe = low;
     }
     // The built-in in-tile switch point counts evaluations per 64-row tile.
-    const int eval_max = tu.eval_max > 0 ? tu.eval_max : default_eval_max(beta) * (fe->RN / 64);
+    const int eval_max = tu.eval_max > 0 ? tu.eval_max : default_eval_max(beta) * fe->RN / 64;
     const bool per_image_k = n > 1;
     // Layout: image i's canvas at offset off_i of each arena, its bitmap at
     // word bm_off_i of each bitmap arena, its tiles from tile0_i.

@@ -397,3 +397,20 @@ def test_tma_staging_on_and_off_identical(oracle_mod, den, torch_cuda, beta):
                     assert k == k_ref and conv == c_ref and np.array_equal(out, ref), (r, c, tma, host)
     finally:
         den.set_option(hgrms.HGRMS_OPT_TMA, 1)
+
+
+@pytest.mark.parametrize("rows,cols,beta", [(17, 33, 1), (18, 240, 1), (19, 241, 1), (256, 256, 1), (37, 481, 1),
+                                            (20, 240, 2), (21, 239, 2), (321, 481, 2), (26, 241, 3), (27, 480, 3),
+                                            (300, 300, 3), (1026, 960, 1), (1027, 960, 1)])
+def test_low_tiles_of_small_calls(oracle_mod, den, torch_cuda, rows, cols, beta):
+    """Calls of few tiles use 32-row tiles: sizes around their core height and
+    width, every pass count up to the launch's and past it, and the two sides
+    of the line to 64-row tiles (1026 x 960, beta 1: 228 tiles of 18 rows)."""
+    img = synth.noisy_image(rows, cols, 0.3, rows * 7 + cols)[1]
+    T = {1: 8, 2: 4, 3: 2}[beta]
+    for max_k in ((1, T - 1, T, T + 1, 32) if rows < 300 else (T, 32)):
+        assert_same(oracle_mod, den, torch_cuda, img, 10, beta, max_k)
+        assert_same(oracle_mod, den, torch_cuda, img, 10, beta, max_k, list_cap=60)
+    low, sms = 32 - 2 * (T - 1) * beta, torch_cuda.cuda.get_device_properties(0).multi_processor_count
+    tiles = -(-rows // low) * -(-cols // 240)
+    assert den.stats()["tile_rows"] == (low if tiles <= 3 * sms // 2 else 64 - 2 * (T - 1) * beta)
