@@ -80,13 +80,17 @@ constexpr int kListThreads = 512;
 // Nothing a pass reads through L1 is written during the same pass; the output
 // canvas, which a pass reads and writes, is read from L2 (__ldcg).
 
-// Bits [start, start + 32) of a bitmap row (outside [0, 32 * nwords): 0).
+// Bits [start, start + N) of a bitmap row in the low bits (outside [0, 32 *
+// nwords): 0; bits from N on are not defined).  The second word is loaded only
+// where the bits reach it.
+template <int N>
 __device__ __forceinline__ uint32_t row_bits(const uint32_t* __restrict__ row, int nwords, int start) {
+    static_assert(N <= 32, "one word of bits");
     const int w0 = start >= 0 ? (start >> 5) : -((31 - start) >> 5);
     const int sh = start - 32 * w0;
     const uint32_t a = (w0 >= 0 && w0 < nwords) ? __ldca(row + w0) : 0u;
-    const uint32_t b = (w0 + 1 >= 0 && w0 + 1 < nwords) ? __ldca(row + w0 + 1) : 0u;
-    return sh ? ((a >> sh) | (b << (32 - sh))) : a;
+    const uint32_t b = (sh > 32 - N && w0 + 1 >= 0 && w0 + 1 < nwords) ? __ldca(row + w0 + 1) : 0u;
+    return __funnelshift_r(a, b, (uint32_t)sh);
 }
 
 // Algorithm 2 for an interior pixel (card <= 2 is implied by flag >
@@ -225,17 +229,19 @@ __device__ __forceinline__ bool grid_barrier(GridBar* b, Ctrl* c, unsigned nbloc
 }
 
 // W bytes of a canvas row starting at p, realigned into ((W + 3) / 4)
-// words (byte j at bits 8 (j % 4) of word j / 4); reads whole aligned words,
-// which the canvas padding keeps in bounds.
+// words (byte j at bits 8 (j % 4) of word j / 4; bytes from W on are not
+// defined); reads whole aligned words, which the canvas padding keeps in
+// bounds, and no more of them than can hold the W bytes (for beta 2 two
+// instead of three: the passes of long lists are bound by their loads).
 template <int W>
 __device__ __forceinline__ void load_row_bytes(const uint8_t* p, uint32_t (&r)[(W + 3) / 4]) {
-    constexpr int NW = (W + 3) / 4;
+    constexpr int NW = (W + 3) / 4, NL = (W + 3 + 3) / 4;
     const uintptr_t a = reinterpret_cast<uintptr_t>(p);
     const uint32_t* q = reinterpret_cast<const uint32_t*>(a & ~uintptr_t(3));
     const uint32_t sh = (uint32_t)(a & 3u) * 8u;
     uint32_t w[NW + 1];
 #pragma unroll
-    for (int i = 0; i <= NW; ++i) w[i] = __ldca(q + i);
+    for (int i = 0; i <= NW; ++i) w[i] = i < NL ? __ldca(q + i) : 0u;
 #pragma unroll
     for (int i = 0; i < NW; ++i) r[i] = __funnelshift_r(w[i], w[i + 1], sh);
 }
@@ -253,7 +259,7 @@ __device__ __forceinline__ void mark_image(uint32_t* bits, bool ch, unsigned img
 __device__ __forceinline__ uint32_t load3_cg(const uint8_t* p) {
     const uintptr_t a = reinterpret_cast<uintptr_t>(p);
     const uint32_t* q = reinterpret_cast<const uint32_t*>(a & ~uintptr_t(3));
-    return __funnelshift_r(__ldcg(q), __ldcg(q + 1), (uint32_t)(a & 3u) * 8u);
+    return __funnelshift_r(__ldcg(q), (a & 3u) > 1u ? __ldcg(q + 1) : 0u, (uint32_t)(a & 3u) * 8u);
 }
 
 // Warp-collective: img_n[img] += d for every lane with d != 0 (one atomic per
@@ -636,7 +642,7 @@ __global__ void __launch_bounds__(kListThreads, 2) list_loop_kernel(PassArgs a) 
                         load_row_bytes<W>(in + off + (long long)(r - B) * d.pitch - B, win[r]);
                         const int gy = qy - B + r;
                         if (gy <= py) {
-                            const uint32_t bits = row_bits(bmp + (size_t)gy * d.bm_words, d.bm_words, qx - B) & ((1u << W) - 1u);
+                            const uint32_t bits = row_bits<W>(bmp + (size_t)gy * d.bm_words, d.bm_words, qx - B) & ((1u << W) - 1u);
                             ahead |= gy < py ? bits : bits & ((1u << (px - qx + B)) - 1u);
                         }
                     }
@@ -690,7 +696,7 @@ __global__ void __launch_bounds__(kListThreads, 2) list_loop_kernel(PassArgs a) 
 #pragma unroll
                     for (int r = 0; r < 3; ++r) {
                         const int gy = py - 2 + r;
-                        rb[r] = gy >= 0 ? row_bits(bmp + (size_t)gy * d.bm_words, d.bm_words, px - 2) : 0u;
+                        rb[r] = gy >= 0 ? row_bits<5>(bmp + (size_t)gy * d.bm_words, d.bm_words, px - 2) : 0u;
                     }
                     // Rows py - 2 .. py + 2, bytes px - 2 .. px + 2 (the canvas padding keeps them in bounds).
                     uint32_t nb[5][2], ob[3];
@@ -777,7 +783,7 @@ __global__ void __launch_bounds__(kListThreads, 2) list_loop_kernel(PassArgs a) 
 #pragma unroll
                         for (int r = 0; r <= 2 * B; ++r) {
                             const int gy = qy - B + r;
-                            rb[r] = (gy <= py) ? row_bits(bmp + (size_t)gy * d.bm_words, d.bm_words, px - 2 * B) : 0u;
+                            rb[r] = (gy <= py) ? row_bits<4 * B + 1>(bmp + (size_t)gy * d.bm_words, d.bm_words, px - 2 * B) : 0u;
                         }
                         uint32_t ahead = 0u;
 #pragma unroll
