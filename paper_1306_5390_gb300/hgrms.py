@@ -10,7 +10,9 @@ from __future__ import annotations
 
 import ctypes
 import os
+import sys
 import threading
+from array import array
 
 import numpy as np
 
@@ -204,15 +206,23 @@ def hgrms_wait(h) -> int:
     return load_library().hgrms_wait(h)
 
 
+def _image_arrays(ptrs, rows, cols):
+    """C arrays of n image pointers and sizes (array fills them at a few ns a
+    value, a ctypes array's constructor at a tenth of a microsecond)."""
+    n = len(ptrs)
+    if n == 0:
+        return (ctypes.c_void_p * 1)(), (ctypes.c_int * 1)(), (ctypes.c_int * 1)()
+    return ((ctypes.c_void_p * n).from_buffer(array("Q", [p or 0 for p in ptrs])), (ctypes.c_int * n).from_buffer(array("i", rows)),
+            (ctypes.c_int * n).from_buffer(array("i", cols)))
+
+
 def hgrms_denoise_batch(h, ptrs, rows, cols, alpha: int, beta: int, max_k: int, k_out) -> int:
     n = len(ptrs)
-    P = (ctypes.c_void_p * max(n, 1))(*ptrs)
-    R = (ctypes.c_int * max(n, 1))(*rows)
-    C = (ctypes.c_int * max(n, 1))(*cols)
+    P, R, C = _image_arrays(ptrs, rows, cols)
     K = (ctypes.c_int * max(n, 1))()
     rc = load_library().hgrms_denoise_batch(h, P, R, C, n, alpha, beta, max_k, K)
-    for i in range(n):
-        k_out[i] = K[i]
+    for i, k in enumerate(K[:n]):
+        k_out[i] = k
     return rc
 
 
@@ -316,6 +326,25 @@ class Denoiser:
             raise ValueError("image must be a contiguous 2-D uint8 tensor")
         return img.data_ptr(), img.shape[0], img.shape[1]
 
+    @staticmethod
+    def _ptrs_shapes(imgs):
+        """([pointer], [rows], [cols]) of many images; the checks of
+        ``_ptr_shape`` in one loop (a batch waits for it before its first
+        launch)."""
+        torch = sys.modules.get("torch")
+        u8, tensor = (torch.uint8, torch.Tensor) if torch is not None else (None, ())
+        ptrs, rows, cols = [], [], []
+        for img in imgs:
+            if isinstance(img, tensor) and img.dtype is u8 and img.dim() == 2 and img.is_contiguous():
+                p = img.data_ptr()
+                r, c = img.shape
+            else:
+                p, r, c = Denoiser._ptr_shape(img)
+            ptrs.append(p)
+            rows.append(r)
+            cols.append(c)
+        return ptrs, rows, cols
+
     def denoise(self, img, alpha: int, beta: int, max_k: int) -> int:
         """Denoise ``img`` in place; returns k.  ``img``: numpy (host) or CUDA tensor."""
         ptr, rows, cols = self._ptr_shape(img)
@@ -341,10 +370,9 @@ class Denoiser:
         return k
 
     def denoise_batch(self, imgs, alpha: int, beta: int, max_k: int):
-        ps = [self._ptr_shape(im) for im in imgs]
-        ks = [0] * len(ps)
-        rc = hgrms_denoise_batch(self.h, [p[0] for p in ps], [p[1] for p in ps], [p[2] for p in ps],
-                                 alpha, beta, max_k, ks)
+        ptrs, rows, cols = self._ptrs_shapes(imgs)
+        ks = [0] * len(ptrs)
+        rc = hgrms_denoise_batch(self.h, ptrs, rows, cols, alpha, beta, max_k, ks)
         if rc != HGRMS_OK:
             raise HgrmsError(rc, "hgrms_denoise_batch")
         return ks
@@ -400,16 +428,14 @@ class Denoiser:
     def predict_k(self, beta: int, imgs, features: bool = False):
         """Predicted k per image (device-readable images); with features=True
         also (x0 [n,64,64], hist [n,16], gap [n,16])."""
-        ps = [self._ptr_shape(im) for im in imgs]
-        n = len(ps)
+        ptrs, rows, cols = self._ptrs_shapes(imgs)
+        n = len(ptrs)
         kh = np.zeros(n, dtype=np.float32)
         fp = ctypes.POINTER(ctypes.c_float)
         x0 = np.zeros((n, 64, 64), dtype=np.float32) if features else None
         hist = np.zeros((n, 16), dtype=np.float32) if features else None
         gap = np.zeros((n, 16), dtype=np.float32) if features else None
-        arr = (ctypes.c_void_p * max(1, n))(*[p[0] for p in ps])
-        rows = (ctypes.c_int * max(1, n))(*[p[1] for p in ps])
-        cols = (ctypes.c_int * max(1, n))(*[p[2] for p in ps])
+        arr, rows, cols = _image_arrays(ptrs, rows, cols)
 
         def ptr(a):
             return a.ctypes.data_as(fp) if a is not None else None

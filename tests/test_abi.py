@@ -6,6 +6,7 @@ import os
 import re
 import subprocess
 
+import numpy as np
 import pytest
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
@@ -136,3 +137,23 @@ def test_header_constants_match_the_binding():
     m = re.search(r"#define\s+HGRMS_NOALLOC_SCRATCH_BYTES\s+\((\d+)u << (\d+)\)", text)
     assert m and hgrms.HGRMS_NOALLOC_SCRATCH_BYTES == int(m.group(1)) << int(m.group(2))
     assert found >= 20
+
+
+def test_batch_marshalling_matches_the_single_image_checks():
+    """The batch loop gives the pointers and sizes of _ptr_shape and refuses
+    what it refuses, for numpy arrays and tensors in any order; a null pointer
+    stays one."""
+    torch = pytest.importorskip("torch")
+    from paper_1306_5390_gb300 import hgrms
+    one = hgrms.Denoiser._ptr_shape
+    a, t = np.zeros((3, 5), np.uint8), torch.zeros((4, 6), dtype=torch.uint8)
+    imgs = [a, t, t[1:], np.zeros((0, 4), np.uint8), t.view(2, 12)]
+    ptrs, rows, cols = hgrms.Denoiser._ptrs_shapes(imgs)
+    assert list(zip(ptrs, rows, cols)) == [one(i) for i in imgs]
+    P, R, C = hgrms._image_arrays(ptrs[:2] + [None], rows[:3], cols[:3])
+    assert list(P) == [a.ctypes.data, t.data_ptr(), None] and list(R) == [3, 4, 3] and list(C) == [5, 6, 6]
+    for bad in (t.t(), t.float(), torch.zeros(3, dtype=torch.uint8), np.zeros((2, 2)), a.T, torch.zeros((2, 2, 2), dtype=torch.uint8)):
+        with pytest.raises(ValueError):
+            one(bad)
+        with pytest.raises(ValueError):
+            hgrms.Denoiser._ptrs_shapes([t, bad])
