@@ -185,11 +185,21 @@ namespace {
 // list pass would evaluate more than 2.5 % of the pixels.  With
 // HGRMS_OPT_RELAUNCH_PPM set, up to 8 for any alpha and beta.
 constexpr int kDefaultRelaunches = 3;
-// Calls of at least this many pixels use the 128-row tiles (where compiled
-// and they compute fewer rows): measured faster on 8192 x 8192 and on the
-// 629 M-pixel uneven batch; smaller calls keep the 64-row tiles, whose larger
-// tile count spreads better over the SMs.
+// The 128-row tiles (where compiled and they compute fewer rows) serve calls of
+// at least this many pixels: measured faster on 8192 x 8192 and on the 629
+// M-pixel uneven batch.  Smaller calls take them when they fill at least two
+// waves and do not need more waves than the 64-row tiles, two of which share an
+// SM (a last wave of those with at most one tile per SM takes 0.6 of a full
+// one): 64 photographs of 321 x 481 (beta 1, 576 tiles, 4 waves against 4.6)
+// 251 us in the fused launch against 271, 2161 x 3839 152 against 177, 40 of
+// 1000 x 800 610 against 663; but 2048 x 2048 of beta 2 (2 against 1.6) 80
+// against 69 and 3000 x 3000 (3 against 2.6) 121 against 102.
 constexpr long long kTallMinPixels = 32ll << 20;
+bool tall_by_waves(long long tiles64, long long tiles128, int sms) {
+    const long long rest = tiles64 % (2 * sms);
+    const long long tenths64 = tiles64 / (2 * sms) * 10 + (rest == 0 ? 0 : (rest <= sms ? 6 : 10));
+    return tiles128 >= 2 * sms && (tiles128 + sms - 1) / sms * 10 <= tenths64;
+}
 // Calls of at most 3/2 32-row tiles per SM take those: 256 x 256 (30 tiles, 12
 // of 64 rows) 25.6 us in the fused launch against 32.7, 321 x 481 25.6 against
 // 33.8 (beta 1) and 35.8 (beta 2), 800 x 1200 (beta 2, 200 tiles) 33.8 against
@@ -640,7 +650,9 @@ int run_hybrid(hgrms_ctx* h, const BatchImg* im, int n, int alpha, int beta, int
             if (tall) rows128 += tx * ((im[i].rows + tall->TH - 1) / tall->TH) * 128;
             if (low) tiles32 += tx * ((im[i].rows + low->TH - 1) / low->TH);
         }
-        if (tall && px_call >= kTallMinPixels && rows128 < rows64) fe = tall;
+        if (tall && rows128 < rows64 &&
+            (px_call >= kTallMinPixels || tall_by_waves(rows64 / 64, rows128 / 128, h->sms)))
+            fe = tall;
         else if (low && tiles32 <= low_tiles_max(h->sms)) fe = low;
     }
     // The built-in in-tile switch point counts evaluations per 64-row tile.

@@ -287,3 +287,23 @@ def test_batch_mixing_device_pinned_and_pageable(oracle_mod, den, torch_cuda):
             outs_get.append(lambda arr=arr: arr.copy())
     ks = den.denoise_batch(work, 10, 1, 32)
     check(oracle_mod, imgs, [g() for g in outs_get], ks, den.converged(), 10, 1, 32, "mixed memory")
+
+
+@pytest.mark.parametrize("n,rows,cols,beta", [(51, 229, 481, 1), (51, 228, 479, 2), (50, 229, 481, 1)])
+def test_tall_tiles_of_mid_sized_batches(oracle_mod, den, torch_cuda, n, rows, cols, beta):
+    """Batches below 32 Mi pixels on both sides of the wave rule: 51 images of 3
+    x 3 (beta 1) or 2 x 2 tall tiles and 50 of them, against the oracle."""
+    base = [synth.noisy_image(rows, cols, d, 950 + i)[1] for i, d in enumerate((0.1, 0.3, 0.6))]
+    imgs = [base[i % 3] for i in range(n)]
+    outs, ks, _ = run_batch(den, torch_cuda, imgs, 10, beta, 33)
+    refs = [oracle_mod.denoise(im, 10, beta, 33) for im in base]
+    for i, (out, k) in enumerate(zip(outs, ks)):
+        ref, k_ref, _ = refs[i % 3]
+        assert k == k_ref and np.array_equal(out, ref), i
+    sms = torch_cuda.cuda.get_device_properties(0).multi_processor_count
+    T = {1: 8, 2: 4}[beta]
+    tiles = {rn: n * -(-rows // (rn - 2 * (T - 1) * beta)) * -(-cols // 240) for rn in (64, 128)}
+    rest = tiles[64] % (2 * sms)
+    tall = tiles[128] >= 2 * sms and -(-tiles[128] // sms) * 10 <= tiles[64] // (2 * sms) * 10 + (
+        0 if rest == 0 else 6 if rest <= sms else 10) and tiles[128] * 128 < tiles[64] * 64
+    assert den.stats()["tile_rows"] == (128 if tall else 64) - 2 * (T - 1) * beta
