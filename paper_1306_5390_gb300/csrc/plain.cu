@@ -156,12 +156,12 @@ cudaError_t launch_copy_in(const uint8_t* img, int rows, int cols, uint8_t* canv
 // A warp takes a piece of an image row of up to kPieceVecs 16-byte words,
 // aligned in the destination: words whose bytes lie at the same alignment in
 // the canvas (16-byte aligned rows) are moved as they are, others are put
-// together from five 4-byte words by funnel shifts; the ends of the row go
-// byte by byte.  Bound by memory: 8192 x 8192 takes 28 us (134 MB, 4.7 TB/s;
-// pieces of 512 words, a whole row per warp, took 17 us more: too many rows
-// open at once).  128 images of 128..2048 pixels a side, 157 MB, 101 us;
-// a call with them 3.34 -> 3.13 ms, 3839 x 2161 0.163 -> 0.136 ms (every 4-byte
-// word, and every byte of an odd row, used to be gathered by itself).
+// together by funnel shifts from two aligned chunks, the second one the next
+// lane's; the ends of the row go byte by byte.  Bound by memory: 8192 x 8192
+// takes 28 us (134 MB, 4.7 TB/s; a whole row per warp took 17 us more: too many
+// rows open at once).  128 images of 128..2048 pixels a side, 157 MB, 92 us
+// (101 from five 4-byte loads a word, about 330 when every 4-byte word, or
+// every byte of an odd row, was gathered by itself); 3839 x 2161 9 us.
 constexpr int kPieceVecs = 128;
 
 __host__ __device__ inline int row_pieces(int cols) {
@@ -185,14 +185,35 @@ __device__ __forceinline__ void copy_rows(const uint8_t* __restrict__ canvas, lo
 #pragma unroll 4
             for (int v = pc * kPieceVecs + lane; v < v1; v += 32) dv[v] = reinterpret_cast<const uint4*>(src)[v];
         } else {
-            const uint32_t* sw = reinterpret_cast<const uint32_t*>(src + (head & ~3));
+            // Word v's bytes lie in the 16-byte chunks v and v + 1 of the
+            // canvas row: a lane loads chunk v and has the next one from the
+            // next lane (its last lane from the first of the next 32).
+            constexpr int kIt = kPieceVecs / 32;
+            const int v0 = pc * kPieceVecs + lane;
+            const uint4* sv = reinterpret_cast<const uint4*>(src);
+            uint4 c[kIt + 1];
+#pragma unroll
+            for (int i = 0; i <= kIt; ++i) {
+                const int v = i < kIt ? v0 + 32 * i : (pc + 1) * kPieceVecs;
+                c[i] = v <= v1 ? sv[v] : make_uint4(0u, 0u, 0u, 0u);
+            }
             const uint32_t sh = (uint32_t)(head & 3) * 8u;
-#pragma unroll 4
-            for (int v = pc * kPieceVecs + lane; v < v1; v += 32) {
-                const uint32_t* q = sw + 4 * v;
-                const uint32_t w0 = q[0], w1 = q[1], w2 = q[2], w3 = q[3], w4 = q[4];
-                dv[v] = make_uint4(__funnelshift_r(w0, w1, sh), __funnelshift_r(w1, w2, sh),
-                                   __funnelshift_r(w2, w3, sh), __funnelshift_r(w3, w4, sh));
+#pragma unroll
+            for (int i = 0; i < kIt; ++i) {
+                const uint4 x = lane == 0 ? c[i + 1] : c[i];
+                const int from = (lane + 1) & 31;
+                const uint32_t n0 = __shfl_sync(0xffffffffu, x.x, from), n1 = __shfl_sync(0xffffffffu, x.y, from);
+                const uint32_t n2 = __shfl_sync(0xffffffffu, x.z, from), n3 = __shfl_sync(0xffffffffu, x.w, from);
+                uint32_t w0, w1, w2, w3, w4;
+                switch (head >> 2) {  // the same for the whole warp
+                    case 0: w0 = c[i].x, w1 = c[i].y, w2 = c[i].z, w3 = c[i].w, w4 = n0; break;
+                    case 1: w0 = c[i].y, w1 = c[i].z, w2 = c[i].w, w3 = n0, w4 = n1; break;
+                    case 2: w0 = c[i].z, w1 = c[i].w, w2 = n0, w3 = n1, w4 = n2; break;
+                    default: w0 = c[i].w, w1 = n0, w2 = n1, w3 = n2, w4 = n3; break;
+                }
+                if (v0 + 32 * i < v1)
+                    dv[v0 + 32 * i] = make_uint4(__funnelshift_r(w0, w1, sh), __funnelshift_r(w1, w2, sh),
+                                                 __funnelshift_r(w2, w3, sh), __funnelshift_r(w3, w4, sh));
             }
         }
         if (pc == pieces - 1) {
