@@ -367,8 +367,9 @@ typedef struct hgrms_stats {
     int    launches;        /* denoising kernel launches issued */
     int    work_launches;   /* of those, launches that ran at least one pass */
     int    passes;          /* passes needed: k, plus 1 if the call ended on a no-change pass */
-    int    passes_executed; /* passes the launches actually ran (a launch runs whole
-                               groups of T, so this can exceed `passes`) */
+    int    passes_executed; /* passes the launches ran (a launch runs whole groups of T, so
+                               this can exceed `passes`); passes whose result was in its
+                               canvas already, so that nothing was left to evaluate, count */
     int    passes_per_launch; /* fused passes per launch (T) */
     int    tile_rows;       /* core tile height of the kernel used */
     int    tile_cols;       /* core tile width of the kernel used */
@@ -380,7 +381,9 @@ typedef struct hgrms_stats {
     long long evals_fused;  /* pixel evaluations the passes needed, fused tile launches
                                (every image pixel per dense pass, else the pixels within
                                beta of a change of the previous pass) */
-    long long evals_list;   /* the same for list-pass launches */
+    long long evals_list;   /* the same for list-pass launches: the pixels whose window
+                               differs from the one two passes back (or, in their first
+                               passes, one pass back) */
     int    tile_eval_max;   /* in-tile list/dense switch point used (HGRMS_OPT_TILE_EVAL_MAX) */
     int    autotuned;       /* 1 if the tuning came from the autotuner (HGRMS_OPT_AUTOTUNE) */
     double tune_ms;         /* device time the autotuner's trials took in this call (0 when the

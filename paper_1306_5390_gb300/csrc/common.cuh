@@ -23,10 +23,8 @@ constexpr int kMaxBatchImages = 4096;  // images per batched launch (more are sp
 // Iteration state shared by the launches of one denoising call.
 //
 // Three canvases hold images.  `cur` holds the current image I_t.  `aux`
-// holds an image that agrees with I_{t-1} wherever pass t changed nothing
-// (I_{t-1} itself after a one-pass launch); a launch that writes only the
-// pixels that can change (a list pass) writes into `aux`, which then holds
-// I_{t+1} everywhere.
+// holds I_{t-1} (hybrid schedule); a list pass writes the pixels where I_{t+1}
+// differs from I_{t-1} into `aux`, which then holds I_{t+1} everywhere.
 struct Ctrl {
     unsigned k;          // passes so far that changed at least one pixel
     unsigned converged;  // 1 once a pass changed no pixel

@@ -5,15 +5,17 @@
 //   1. host images the device cannot read are copied into canvas A (padded,
 //      16-byte aligned rows); the first fused launch reads the others
 //      (device memory, mapped page-locked host memory) directly,
-//   2. reset the device control block (k = 0, current canvas = A),
+//   2. one launch clears the control block (k = 0, current canvas = A), the
+//      change bitmaps and the barrier,
 //   3. enqueue the passes (Section 2's iteration): by default one fused
 //      launch of T passes on shared-memory tiles of every image (the passes
 //      where many pixels change), then one persistent launch that runs each
-//      remaining pass as a list pass, evaluating only the windows around the
-//      pixels the previous pass changed.  k, the converged flag and the
+//      remaining pass as a list pass, evaluating only the pixels that can
+//      differ from what their canvas holds.  k, the converged flag and the
 //      current canvas are kept on the device, so no launch waits for the
 //      host,
-//   4. copy the current canvas back and read k with one device-to-host copy.
+//   4. one launch copies the current canvas to the caller's image and k and
+//      the control block to page-locked host memory.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 #include <cuda_runtime.h>
