@@ -248,6 +248,32 @@ __device__ __forceinline__ int warp_excl_scan(const int lane, const int n, int* 
     return incl - n;
 }
 
+// Programmatic dependent launches.  A launch made with launch_dependent may
+// become resident before the launch ahead of it in its stream has ended: it
+// must reach wait_for_previous before it touches memory (the wait lasts until
+// that launch has completed and its writes are visible; no-op otherwise).
+// let_next_start, in the launch ahead, allows that from there on.  Used for a
+// call's fused launches (behind the init launch) and its last one: a call loses
+// 3 to 5 us of launch latency (256 x 256 52.5 -> 49.1 us, 3839 x 2161 136 -> 131).
+__device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <class... Params, class... Args>
+cudaError_t launch_dependent(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                             Args&&... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
+}
+
 // Passes the launch must run: 0 when the call has finished.
 __device__ __forceinline__ int launch_passes(const Ctrl* c, int T) {
     unsigned k = __ldcg(&c->k);

@@ -927,6 +927,7 @@ fused_kernel(PassArgs a) {
     const int tid = threadIdx.x;
     const int lane = tid & 31, warp = tid >> 5;
     Ctrl* ctrl = a.ctrl;
+    wait_for_previous();
     if (tid == 0) {
         int np = launch_passes(ctrl, T);
         // Every launch that did work before this one was a fused launch.
@@ -1371,8 +1372,7 @@ cudaError_t launch_fused(const PassArgs& a, int ctas, cudaStream_t s) {
     }
     const long long cap = (long long)sms[dev] * occ[dev];
     const unsigned grid = (unsigned)(ctas < cap ? (ctas > 0 ? ctas : 1) : cap);
-    fused_kernel<B, T, RN><<<grid, G::kThreads, G::kSmem, s>>>(a);
-    return cudaGetLastError();
+    return launch_dependent(fused_kernel<B, T, RN>, dim3(grid), dim3(G::kThreads), G::kSmem, s, a);
 }
 
 template <int B, int T, int RN = 64>

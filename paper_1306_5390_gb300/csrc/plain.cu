@@ -92,6 +92,7 @@ cudaError_t launch_plain(int beta, const PassArgs& a, cudaStream_t s) {
 // each.)
 __global__ void call_init_kernel(Ctrl* __restrict__ c, unsigned max_k, uint4* __restrict__ bm, long long n16,
                                  GridBar* __restrict__ bar, unsigned* __restrict__ counts, long long nk) {
+    let_next_start();
     const long long g = blockIdx.x * (long long)blockDim.x + threadIdx.x, gt = (long long)gridDim.x * blockDim.x;
     if (g == 0) {
         Ctrl z = {};
@@ -225,6 +226,7 @@ __device__ __forceinline__ void copy_rows(const uint8_t* __restrict__ canvas, lo
 }
 
 __global__ void __launch_bounds__(256) call_finish_kernel(FinishArgs a) {
+    wait_for_previous();
     const Ctrl* c = a.ctrl;
     const int lane = threadIdx.x & 31, warp = (blockIdx.x * 256 + threadIdx.x) >> 5, nwarps = gridDim.x * 8;
     const uint8_t* canvas = a.arena[__ldcg(&c->cur)];
@@ -253,8 +255,7 @@ cudaError_t launch_call_finish(const FinishArgs& a, int sms, cudaStream_t s) {
     const unsigned gy = a.imgs ? (unsigned)a.nimg : 1u;
     const long long cap = a.imgs ? std::max(((long long)sms * 16 + gy - 1) / gy, 16ll) : (long long)sms * 8;
     gx = std::min(std::max(gx, 1ll), cap);
-    call_finish_kernel<<<dim3((unsigned)gx, gy), 256, 0, s>>>(a);
-    return cudaGetLastError();
+    return launch_dependent(call_finish_kernel, dim3((unsigned)gx, gy), dim3(256), 0, s, a);
 }
 
 // tile_img[b] = the image that fused tile b belongs to.
