@@ -477,6 +477,7 @@ __global__ void __launch_bounds__(kListThreads, 2) list_loop_kernel(PassArgs a) 
     bool failed = false;
     unsigned evals = 0;
     int qpar = 0;  // queue counter of the next chunk (CTA-uniform)
+    int round = 0;  // entry of ctrl->solo for the next passes of one CTA (the same in every CTA)
     const long long gthreads = (long long)gridDim.x * blockDim.x;
     const long long gtid = (long long)blockIdx.x * blockDim.x + tid;
     const long long warp_base = (long long)blockIdx.x * blockDim.x + (tid & ~31);
@@ -537,9 +538,9 @@ __global__ void __launch_bounds__(kListThreads, 2) list_loop_kernel(PassArgs a) 
                     s_qn[0] = s_qn[1] = 0;
                     if (s_dn) atomicAdd(&ctrl->n_diff, s_dn);
                     s_dn = 0;
-                    ctrl->solo_k = st.k;
-                    ctrl->solo_n = st.n_cur;
-                    ctrl->solo_before = st.c_list ? st.n_before : 0xffffffffu;
+                    ctrl->solo[round].k = st.k;
+                    ctrl->solo[round].n = st.n_cur;
+                    ctrl->solo[round].before = st.c_list ? st.n_before : 0xffffffffu;
                 }
             }
             unsigned zero = 0;
@@ -549,9 +550,9 @@ __global__ void __launch_bounds__(kListThreads, 2) list_loop_kernel(PassArgs a) 
             }
             if (blockIdx.x != 0) {
                 if (tid == 0) {
-                    s_k = __ldcg(&ctrl->solo_k);
-                    s_n = __ldcg(&ctrl->solo_n);
-                    s_nclr = __ldcg(&ctrl->solo_before);
+                    s_k = __ldcg(&ctrl->solo[round].k);
+                    s_n = __ldcg(&ctrl->solo[round].n);
+                    s_nclr = __ldcg(&ctrl->solo[round].before);
                 }
                 __syncthreads();
                 const unsigned ran = s_k - st.k;
@@ -567,6 +568,9 @@ __global__ void __launch_bounds__(kListThreads, 2) list_loop_kernel(PassArgs a) 
                 }
             }
             if (st.n_cur == 0u || st.k >= max_k) break;
+            // The next write of this entry is two rounds away, behind a
+            // barrier that every CTA reaches after its reads above.
+            round ^= 1;
             continue;
         }
         const int si = (st.t + base) & 3, so = (st.t + base + 1) & 3, sc = (st.t + base + 3) & 3;

@@ -28,9 +28,10 @@ def dilate(m, b):
     return out
 
 
-def list_passes(oracle_mod, cur, aux, k, alpha, beta, max_k, c_first_below):
+def list_passes(oracle_mod, cur, aux, k, alpha, beta, max_k, c_first_below, sizes=None):
     """The loop from I_k = cur and I_(k-1) = aux on: (image, k, converged).
-    c_first_below: the first pass makes C when k is below it."""
+    c_first_below: the first pass makes C when k is below it.  sizes, when
+    given, receives the length of the list that each pass reads."""
     rows, cols = cur.shape
     inner = np.zeros((rows, cols), dtype=bool)
     if rows > 2 * beta and cols > 2 * beta:
@@ -38,6 +39,8 @@ def list_passes(oracle_mod, cur, aux, k, alpha, beta, max_k, c_first_below):
     listed, c_list, before, k0, N = cur != aux, True, 0, k, 0
     while True:
         n = int(listed.sum())
+        if sizes is not None:
+            sizes.append(n)
         make_c = c_list and (k0 < c_first_below if before == 0 else n * 5 < before * 3)
         ev = dilate(listed, beta) & inner
         new, _ = oracle_mod.one_pass(cur, alpha, beta)
@@ -171,6 +174,39 @@ def test_batch_k_of_images_that_stop_at_different_passes(oracle_mod, den, torch_
         ref, k_ref, c_ref = oracle_mod.denoise(im, 10, beta, max_k)
         assert k == k_ref and (k < max_k) == c_ref, (i, k, k_ref)
         assert np.array_equal(t.cpu().numpy(), ref), i
+
+
+# Random images whose lists never get empty, by alpha: cycles of 3, 4 and 6
+# passes, each of one to three listed pixels: (seed, rows, columns).
+CYCLES = {2: [(506, 11, 8), (612, 12, 6), (777, 14, 11), (792, 13, 11), (804, 9, 14)],
+          3: [(45, 15, 11), (219, 6, 12), (785, 13, 9), (843, 15, 15)]}
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("more", [0, 1, 2, 3, 1023, 1024, 1025, 3000])
+@pytest.mark.parametrize("alpha", sorted(CYCLES))
+def test_short_lists_that_outlive_a_round_of_one_cta(oracle_mod, den, torch_cuda, alpha, more):
+    """One CTA runs at most 1024 passes before the others hear of them, and at
+    once starts the next round when the list is still short: calls that end
+    with, and a few passes after, the first, second and third round (the
+    fused launch runs 8 passes), one image and all of them, against the
+    oracle."""
+    max_k = 8 + 1024 + more
+    imgs = [synth.random_image(r, c, seed) for seed, r, c in CYCLES[alpha]]
+    refs = [oracle_mod.denoise(im, alpha, 1, max_k) for im in imgs]
+    for im, ref in zip(imgs, refs):
+        assert ref[1] == max_k and not ref[2]
+        assert not np.array_equal(ref[0], oracle_mod.denoise(im, alpha, 1, max_k - 2)[0])  # a list to the end
+    for im, ref in zip(imgs, refs):
+        for _ in range(5):
+            t = torch_cuda.from_numpy(im.copy()).cuda()
+            assert den.denoise(t, alpha, 1, max_k) == max_k and not den.converged()
+            assert np.array_equal(t.cpu().numpy(), ref[0])
+    for _ in range(5):
+        ts = [torch_cuda.from_numpy(im.copy()).cuda() for im in imgs]
+        assert den.denoise_batch(ts, alpha, 1, max_k) == [max_k] * len(imgs) and not den.converged()
+        for t, ref in zip(ts, refs):
+            assert np.array_equal(t.cpu().numpy(), ref[0])
 
 
 @pytest.mark.gpu
