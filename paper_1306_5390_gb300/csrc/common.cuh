@@ -46,9 +46,9 @@ struct Ctrl {
     unsigned long long evals_list;
     // List-pass launch: pixels changed by the last pass it ran, and the state
     // that the passes of one CTA alone leave to the others (k, list length,
-    // length of the list before, or ~0 when the list is a D_t).  Rounds of such
-    // passes alternate between the two entries: nothing but a round's own
-    // barrier lies between one round and the next, so the CTAs may still be
+    // length of the list before, or ~0 when the list is a D_t).  The entry
+    // alternates with the grid barriers: nothing but a round's own barrier lies
+    // between one round of such passes and the next, so the CTAs may still be
     // reading the last round's entry while CTA 0 writes this one's.
     int n_diff;
     struct {

@@ -469,7 +469,7 @@ __global__ void __launch_bounds__(kListThreads, 2) list_loop_kernel(PassArgs a) 
     st.aux = s_aux;
     st.c_list = true;
     st.n_before = 0u;
-    unsigned gen = 0u;                // barriers completed; the barrier struct is zeroed at the start of every call
+    unsigned gen = 0u;               // thread 0: barriers completed; the barrier struct is zeroed at the start of every call
     unsigned prev_hi[2] = {0u, 0u};  // thread 0: counts seen at the last use of each barrier counter
     const int base = (int)s_base;
     const unsigned max_k = s_maxk, k0 = s_k;
@@ -477,7 +477,6 @@ __global__ void __launch_bounds__(kListThreads, 2) list_loop_kernel(PassArgs a) 
     bool failed = false;
     unsigned evals = 0;
     int qpar = 0;  // queue counter of the next chunk (CTA-uniform)
-    int round = 0;  // entry of ctrl->solo for the next passes of one CTA (the same in every CTA)
     const long long gthreads = (long long)gridDim.x * blockDim.x;
     const long long gtid = (long long)blockIdx.x * blockDim.x + tid;
     const long long warp_base = (long long)blockIdx.x * blockDim.x + (tid & ~31);
@@ -538,9 +537,13 @@ __global__ void __launch_bounds__(kListThreads, 2) list_loop_kernel(PassArgs a) 
                     s_qn[0] = s_qn[1] = 0;
                     if (s_dn) atomicAdd(&ctrl->n_diff, s_dn);
                     s_dn = 0;
-                    ctrl->solo[round].k = st.k;
-                    ctrl->solo[round].n = st.n_cur;
-                    ctrl->solo[round].before = st.c_list ? st.n_before : 0xffffffffu;
+                    // The entry of the barrier ahead, by its parity: it is
+                    // written again two barriers on at the earliest, and every
+                    // CTA reaches the one in between after its reads below.
+                    auto& e = ctrl->solo[gen & 1u];
+                    e.k = st.k;
+                    e.n = st.n_cur;
+                    e.before = st.c_list ? st.n_before : 0xffffffffu;
                 }
             }
             unsigned zero = 0;
@@ -550,9 +553,10 @@ __global__ void __launch_bounds__(kListThreads, 2) list_loop_kernel(PassArgs a) 
             }
             if (blockIdx.x != 0) {
                 if (tid == 0) {
-                    s_k = __ldcg(&ctrl->solo[round].k);
-                    s_n = __ldcg(&ctrl->solo[round].n);
-                    s_nclr = __ldcg(&ctrl->solo[round].before);
+                    const auto& e = ctrl->solo[(gen & 1u) ^ 1u];  // the barrier counted itself
+                    s_k = __ldcg(&e.k);
+                    s_n = __ldcg(&e.n);
+                    s_nclr = __ldcg(&e.before);
                 }
                 __syncthreads();
                 const unsigned ran = s_k - st.k;
@@ -568,9 +572,6 @@ __global__ void __launch_bounds__(kListThreads, 2) list_loop_kernel(PassArgs a) 
                 }
             }
             if (st.n_cur == 0u || st.k >= max_k) break;
-            // The next write of this entry is two rounds away, behind a
-            // barrier that every CTA reaches after its reads above.
-            round ^= 1;
             continue;
         }
         const int si = (st.t + base) & 3, so = (st.t + base + 1) & 3, sc = (st.t + base + 3) & 3;
