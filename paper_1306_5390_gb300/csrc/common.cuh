@@ -18,6 +18,7 @@ namespace hg {
 constexpr int kPadX = 16;   // bytes left of the image; keeps rows 16-byte aligned
 constexpr int kPadY = 16;   // rows above the image (>= any vertical tile halo)
 constexpr int kMaxBeta = 7;
+constexpr unsigned kShortList = 4096;  // change lists up to this cost a list pass its latency, hardly more
 constexpr int kMaxBatchImages = 4096;  // images per batched launch (more are split into chunks)
 
 // Iteration state shared by the launches of one denoising call.
@@ -126,6 +127,7 @@ struct PassArgs {
     // (t + 1) % 4 and clears bitmap (t + 3) % 4.  Null when unused.
     uint32_t* lists[4];
     unsigned list_cap;
+    unsigned list_dense;      // longer lists count as dense (list passes: which list a pass makes, and how)
     uint32_t* bitmaps[4];
     int bm_words;
     int write_prev;           // fused kernel: also write I_{t-1} to the third canvas

@@ -22,13 +22,18 @@
 // It serves as well (a pixel with no such p in its window keeps I_t(q) =
 // I_(t-1)(q)), and a pass that reads C_t finds every pixel of C_(t+1) and of
 // D_(t+1) and can make either; a pass that reads D_t can make only D_(t+1).  D_t
-// holds C_(t-1)'s settled pixels too, so while the changes still die out
-// quickly C is the shorter list.  A pass therefore makes C again while
-// the last list was shorter than 3/5 of the one before it (beta 5, 1000 x
+// holds C_(t-1)'s settled pixels too, so while the changes still die out C is the
+// shorter list.  make_c draws the line: C again while the last list was
+// shorter than 3/4 (short lists 3/5) of the one before it (beta 5, 1000 x
 // 1500, 2 % impulses: 1.5 M evaluations against 2.8 M with D from the first
 // pass on); the first pass, which knows no ratio, makes D when the fused
 // launches ran kDirectD passes, by then the changes left are mostly
-// oscillations.
+// oscillations.  Lists of more than 1/32 of the pixels are no oscillations
+// yet: they make C while they shrink at all (textured 4096 x 4096, 70 %
+// impulses, beta 3: alpha 1 4.17 ms a call against 5.16 when D began at once, alpha
+// 2 1.75 against 2.15; 8192 x 8192, alpha 2, beta 1: 6.5 against 7.4), and with
+// alpha 0, which replaces every interior pixel in every pass, however they
+// shrink (1024 x 1024, beta 1: 0.64 ms against 0.75).
 //
 // k and the converged flag need to know whether a pass changed the image,
 // N_t = #{q : I_t(q) != I_(t-1)(q)} > 0.  For a pixel that is not evaluated
@@ -301,10 +306,13 @@ struct LoopState {
     unsigned n_last;    // entries of the list before it (its bitmap is cleared by the next pass)
     unsigned n_before;  // entries of the list that the last pass read (0: no pass yet)
     bool c_list;        // the next pass reads C_t (else D_t)
-    // Whether the next pass, from a list of n entries, makes C (see the header; k0: passes before this launch).
-    __device__ __forceinline__ bool make_c(unsigned n, unsigned k0) const {
-        return c_list && (n_before == 0u ? k0 < kDirectD
-                                         : (unsigned long long)n * 5u < (unsigned long long)n_before * 3u);
+    // Whether the next pass, from a list of n entries, makes C (see the header;
+    // k0: passes before this launch, dense: 1/32 of the pixels).
+    __device__ __forceinline__ bool make_c(unsigned n, unsigned k0, unsigned dense, int alpha) const {
+        if (!c_list) return false;
+        const unsigned long long now = n, before = n_before;
+        if (n > dense && (n_before == 0u || now * 16u < before * 15u || (alpha == 0 && n / 4u > dense))) return true;
+        return n_before == 0u ? k0 < kDirectD : (n > kShortList ? now * 4u < before * 3u : now * 5u < before * 3u);
     }
 };
 
@@ -352,7 +360,7 @@ __device__ __forceinline__ void solo_passes(const PassArgs& a, const ImgDesc& on
         const uint8_t* in_arena = a.canvas[st.cur];
         uint8_t* out_arena = a.canvas[st.aux];
         const int ntask = (int)n * P;
-        const bool make_c = st.make_c(n, k0);
+        const bool make_c = st.make_c(n, k0, a.list_dense, a.alpha);
         for (int i = tid; i < ntask; i += kListThreads) {
             const int e = i / P, o = i - e * P;
             unsigned img;
@@ -582,22 +590,26 @@ __global__ void __launch_bounds__(kListThreads, 2) list_loop_kernel(PassArgs a) 
         uint32_t* next = a.lists[so];
         uint32_t* bm_next = a.bitmaps[so];
         unsigned* nnext = &ctrl->list_n[so];
-        const bool make_c = st.make_c(st.n_cur, k0);
+        const bool make_c = st.make_c(st.n_cur, k0, a.list_dense, a.alpha);
         // N is needed from the first D_t on: the pass that makes it counts the
         // pixels it changes, the later ones the differences.
         const int add = make_c ? 0 : 1, sub = st.c_list ? 0 : 1;
+        const bool blind = make_c && st.c_list;
         if (tid == 0 && blockIdx.x == 0) {
             // Set (t + base + 2) % 4 is next written by pass t + 1; its list
             // was last read (to clear its bitmap) in pass t - 1.
             ctrl->list_n[(st.t + base + 2) & 3] = 0u;
         }
         const unsigned n = st.n_cur, nclr = st.n_last;
+        // The windows of an eighth of the pixels hold nearly all of them: for
+        // beta >= 2 a pass over every pixel costs less than one by such a list.
+        const bool whole = n > a.list_cap || (B > 1 && n / 4u > a.list_dense);
         // A short list: one thread per (listed pixel, window position).
-        const bool direct = B <= kDirectB && (long long)n * P <= gthreads && n <= a.list_cap;
+        const bool direct = B <= kDirectB && (long long)n * P <= gthreads && !whole;
         // The list entry of this thread's first task, loaded before the bitmap clearing below so that the two
         // loads overlap.
         uint32_t pk_first = 0u;
-        if (n <= a.list_cap) {
+        if (!whole) {
             const long long i0 = first_task;
             const long long per = direct ? P : (B == 1 ? 1 : W);
             if (i0 < (long long)n * per) pk_first = __ldcg(prev + (unsigned)(i0 / per));
@@ -674,7 +686,7 @@ __global__ void __launch_bounds__(kListThreads, 2) list_loop_kernel(PassArgs a) 
                 add_image(a.img_n, delta, img, lane);
             }
             staged_append(sl, next, nnext, a.list_cap, ch, v, lane);
-        } else if (n <= a.list_cap && B == 1) {
+        } else if (!whole && B == 1) {
             // beta 1: one thread per listed pixel p.  It loads p's 5 x 5
             // neighbourhood, the 3 x 3 window of the output canvas and the
             // list's bits of the rows up to p's, and evaluates every pixel q
@@ -757,7 +769,7 @@ __global__ void __launch_bounds__(kListThreads, 2) list_loop_kernel(PassArgs a) 
                 });
                 pk = pk_next;
             }
-        } else if (n <= a.list_cap) {
+        } else if (!whole) {
             // Chunks of one task per thread: task (listed pixel p, window
             // row dy) finds the pixels q = p + (dy, dx) that p owns and
             // queues them in shared memory (phase A); the CTA then evaluates
@@ -873,7 +885,7 @@ __global__ void __launch_bounds__(kListThreads, 2) list_loop_kernel(PassArgs a) 
                 pk = pk_next;
             }
         } else {
-            // The list overflowed: evaluate every pixel of every image.
+            // Evaluate every pixel of every image.
             for (int im = 0; im < (kBatch ? a.nimg : 1); ++im) {
                 const ImgDesc d = kBatch ? load_desc(a.imgs, (unsigned)im) : one;
                 const uint8_t* in = in_arena + d.off + (long long)kPadY * d.pitch + kPadX;
@@ -887,11 +899,12 @@ __global__ void __launch_bounds__(kListThreads, 2) list_loop_kernel(PassArgs a) 
                         const int y = (int)(i / d.cols), x = (int)(i - (long long)y * d.cols);
                         const long long off = (long long)y * d.pitch + x;
                         ++evals;
-                        const int ip = in[off], was = __ldcg(out + off);
+                        // From C to C what the output holds does not matter: it is written over unread.
+                        const int ip = in[off], was = blind ? ip : __ldcg(out + off);
                         int nv = ip;
                         if (y >= B && y < d.rows - B && x >= B && x < d.cols - B)
                             nv = eval_pixel<B>(in + off, d.pitch, a.alpha);
-                        if (nv != was) out[off] = (uint8_t)nv;
+                        if (blind || nv != was) out[off] = (uint8_t)nv;
                         if (nv != (make_c ? ip : was)) {
                             ch = true;
                             v = pack_entry((unsigned)im, y, x, xb, yb);

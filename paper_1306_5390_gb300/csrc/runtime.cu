@@ -728,6 +728,7 @@ int run_hybrid(hgrms_ctx* h, const BatchImg* im, int n, int alpha, int beta, int
         a.bitmaps[i] = h->bitmaps + i * (size_t)bm_total;
     }
     a.list_cap = (unsigned)list_cap;
+    a.list_dense = (unsigned)std::max(px_total / 32, (long long)hg::kShortList);
     a.bm_words = h->host_desc[0].bm_words;
     a.write_prev = 1;
     a.bar = h->bar;

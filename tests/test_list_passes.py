@@ -28,10 +28,21 @@ def dilate(m, b):
     return out
 
 
-def list_passes(oracle_mod, cur, aux, k, alpha, beta, max_k, c_first_below, sizes=None):
+def makes_c(n, before, alpha, k0, c_first_below, dense, short):
+    """Whether a pass that reads a list C of n pixels makes C again (before: the
+    length of the list before it, 0 for the first pass)."""
+    if n > dense and (before == 0 or n * 16 < before * 15 or (alpha == 0 and n // 4 > dense)):
+        return True
+    if before == 0:
+        return k0 < c_first_below
+    return n * 4 < before * 3 if n > short else n * 5 < before * 3
+
+
+def list_passes(oracle_mod, cur, aux, k, alpha, beta, max_k, c_first_below, sizes=None, dense=1 << 30, short=4096):
     """The loop from I_k = cur and I_(k-1) = aux on: (image, k, converged).
-    c_first_below: the first pass makes C when k is below it.  sizes, when
-    given, receives the length of the list that each pass reads."""
+    c_first_below: the first pass makes C when k is below it; longer lists than
+    dense and short follow other lines.  sizes, when given, receives the length
+    of the list that each pass reads."""
     rows, cols = cur.shape
     inner = np.zeros((rows, cols), dtype=bool)
     if rows > 2 * beta and cols > 2 * beta:
@@ -41,7 +52,7 @@ def list_passes(oracle_mod, cur, aux, k, alpha, beta, max_k, c_first_below, size
         n = int(listed.sum())
         if sizes is not None:
             sizes.append(n)
-        make_c = c_list and (k0 < c_first_below if before == 0 else n * 5 < before * 3)
+        make_c = c_list and makes_c(n, before, alpha, k0, c_first_below, dense, short)
         ev = dilate(listed, beta) & inner
         new, _ = oracle_mod.one_pass(cur, alpha, beta)
         out = np.where(ev, new, aux)  # a pixel that is not evaluated keeps what the output holds
@@ -81,10 +92,10 @@ def test_rules_give_the_oracles_iteration(oracle_mod, beta):
         aux, cur = img, img
         for k0 in range(1, min(k_ref, max_k - 1) + 1):
             aux, cur = cur, oracle_mod.one_pass(cur, alpha, beta)[0]
-            for below in (0, 99):
-                out, k, c = list_passes(oracle_mod, cur, aux, k0, alpha, beta, max_k, below)
+            for below, dense, short in ((0, 1 << 30, 4096), (99, 1 << 30, 4096), (0, 4, 4), (6, 16, 0), (0, 0, 0)):
+                out, k, c = list_passes(oracle_mod, cur, aux, k0, alpha, beta, max_k, below, dense=dense, short=short)
                 assert (k, c) == (k_ref, c_ref) and np.array_equal(out, ref), (trial, rows, cols, alpha, max_k, k0,
-                                                                               below, k, k_ref)
+                                                                               below, dense, short, k, k_ref)
             seen.add((bool(c_ref), k_ref == max_k))
     assert {(True, False), (False, True)} <= seen
 
@@ -174,6 +185,37 @@ def test_batch_k_of_images_that_stop_at_different_passes(oracle_mod, den, torch_
         ref, k_ref, c_ref = oracle_mod.denoise(im, 10, beta, max_k)
         assert k == k_ref and (k < max_k) == c_ref, (i, k, k_ref)
         assert np.array_equal(t.cpu().numpy(), ref), i
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("alpha,beta", [(0, 1), (1, 1), (2, 1), (0, 2), (1, 2), (2, 2), (0, 3), (1, 3), (0, 5)])
+def test_dense_lists(oracle_mod, den, torch_cuda, alpha, beta):
+    """Lists of more than 1/32 and 1/8 of the pixels, with and without
+    overflow, down to short ones: one image and a batch, from one fused pass on."""
+    from paper_1306_5390_gb300 import hgrms
+    clean = synth.noisy_image(403, 517, 0.0, 81)[1].astype(np.int64)
+    rng = np.random.default_rng(82)
+    img = np.clip(clean + rng.integers(-8, 9, clean.shape), 0, 255).astype(np.uint8)
+    u = rng.random(img.shape)
+    img[u < 0.3], img[u > 0.7] = 0, 255
+    imgs = [img, np.ascontiguousarray(img[:150, :301]), np.ascontiguousarray(img[::-1])]
+    refs = [oracle_mod.denoise(im, alpha, beta, 27) for im in imgs]
+    first, n = oracle_mod.one_pass(img, alpha, beta)
+    assert n > img.size // 8 and n > 4096
+    for cap in (0, 1 << 20):
+        den.set_option(hgrms.HGRMS_OPT_PASSES, 1)
+        den.set_option(hgrms.HGRMS_OPT_LIST_CAP, cap)
+        try:
+            t = torch_cuda.from_numpy(img.copy()).cuda()
+            k, conv = den.denoise(t, alpha, beta, 27), den.converged()
+            ts = [torch_cuda.from_numpy(im.copy()).cuda() for im in imgs]
+            ks = den.denoise_batch(ts, alpha, beta, 27)
+        finally:
+            den.set_option(hgrms.HGRMS_OPT_PASSES, 0)
+            den.set_option(hgrms.HGRMS_OPT_LIST_CAP, 0)
+        assert (k, conv) == refs[0][1:] and np.array_equal(t.cpu().numpy(), refs[0][0])
+        for t, k, ref in zip(ts, ks, refs):
+            assert k == ref[1] and np.array_equal(t.cpu().numpy(), ref[0])
 
 
 # Random images whose lists never get empty, by alpha: cycles of 3, 4 and 6
