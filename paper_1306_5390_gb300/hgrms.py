@@ -207,18 +207,31 @@ def hgrms_wait(h) -> int:
 
 
 def _image_arrays(ptrs, rows, cols):
-    """C arrays of n image pointers and sizes (array fills them at a few ns a
-    value, a ctypes array's constructor at a tenth of a microsecond)."""
+    """C arrays of n image pointers and sizes from lists of n whole numbers each
+    (array fills them at a few ns a value, a ctypes array's constructor at a
+    tenth of a microsecond)."""
     n = len(ptrs)
-    if n == 0:
-        return (ctypes.c_void_p * 1)(), (ctypes.c_int * 1)(), (ctypes.c_int * 1)()
-    return ((ctypes.c_void_p * n).from_buffer(array("Q", [p or 0 for p in ptrs])), (ctypes.c_int * n).from_buffer(array("i", rows)),
-            (ctypes.c_int * n).from_buffer(array("i", cols)))
+    try:
+        if n > 0:
+            return ((ctypes.c_void_p * n).from_buffer(array("Q", [p or 0 for p in ptrs])),
+                    (ctypes.c_int * n).from_buffer(array("i", rows)), (ctypes.c_int * n).from_buffer(array("i", cols)))
+    except OverflowError:
+        pass  # a size that ctypes cuts to 32 bits: the library sees what a single image's call shows it
+    return _ctypes_arrays(ptrs, rows, cols)
+
+
+def _ctypes_arrays(ptrs, rows, cols):
+    """The same from anything that ctypes takes for them."""
+    n = max(len(ptrs), 1)
+    return (ctypes.c_void_p * n)(*ptrs), (ctypes.c_int * n)(*rows), (ctypes.c_int * n)(*cols)
 
 
 def hgrms_denoise_batch(h, ptrs, rows, cols, alpha: int, beta: int, max_k: int, k_out) -> int:
-    n = len(ptrs)
-    P, R, C = _image_arrays(ptrs, rows, cols)
+    return _denoise_batch(h, len(ptrs), _ctypes_arrays(ptrs, rows, cols), alpha, beta, max_k, k_out)
+
+
+def _denoise_batch(h, n, images, alpha, beta, max_k, k_out) -> int:
+    P, R, C = images
     K = (ctypes.c_int * max(n, 1))()
     rc = load_library().hgrms_denoise_batch(h, P, R, C, n, alpha, beta, max_k, K)
     for i, k in enumerate(K[:n]):
@@ -372,7 +385,7 @@ class Denoiser:
     def denoise_batch(self, imgs, alpha: int, beta: int, max_k: int):
         ptrs, rows, cols = self._ptrs_shapes(imgs)
         ks = [0] * len(ptrs)
-        rc = hgrms_denoise_batch(self.h, ptrs, rows, cols, alpha, beta, max_k, ks)
+        rc = _denoise_batch(self.h, len(ptrs), _image_arrays(ptrs, rows, cols), alpha, beta, max_k, ks)
         if rc != HGRMS_OK:
             raise HgrmsError(rc, "hgrms_denoise_batch")
         return ks

@@ -157,3 +157,40 @@ def test_batch_marshalling_matches_the_single_image_checks():
             one(bad)
         with pytest.raises(ValueError):
             hgrms.Denoiser._ptrs_shapes([t, bad])
+
+
+class FakeLibrary:
+    """Records the images of a batch call."""
+
+    def hgrms_denoise_batch(self, h, P, R, C, n, alpha, beta, max_k, K):
+        self.images = list(P), list(R), list(C), n
+        return 0
+
+
+def test_raw_batch_call_converts_as_ctypes_does(monkeypatch):
+    """The raw call takes and refuses what ctypes arrays of the images' pointers
+    and sizes take and refuse."""
+    from paper_1306_5390_gb300 import hgrms
+    lib = FakeLibrary()
+    monkeypatch.setattr(hgrms, "load_library", lambda: lib)
+
+    def call(ptrs, rows, cols):
+        return hgrms.hgrms_denoise_batch(None, ptrs, rows, cols, 10, 1, 5, [0] * len(ptrs))
+    assert call([ctypes.c_void_p(64), None, 80], (r for r in (1, ctypes.c_int(2), 3)), (4, True, 6)) == 0
+    assert lib.images == ([64, None, 80], [1, 2, 3], [4, 1, 6], 3)
+    call([64, -1], [1], [2 ** 32 + 5, 7])  # missing sizes are 0, which the library refuses
+    assert lib.images == ([64, ctypes.c_void_p(-1).value], [1, 0], [5, 7], 2)
+    call([], [], [])
+    assert lib.images == ([None], [0], [0], 0)
+    for ptrs, rows, cols in (([64], [1, 2], [3]), ([64], [1], [3, 4])):
+        with pytest.raises(IndexError):
+            call(ptrs, rows, cols)
+    for ptrs, rows, cols in ((["64"], [1], [3]), ([64], [1.0], [3])):
+        with pytest.raises(TypeError):
+            call(ptrs, rows, cols)
+
+
+def test_batch_sizes_past_32_bits_reach_the_library_as_a_single_images_do():
+    from paper_1306_5390_gb300 import hgrms
+    P, R, C = hgrms._image_arrays([64, 80], [1, 2], [2 ** 32 + 5, 2 ** 31])
+    assert (list(P), list(R), list(C)) == ([64, 80], [1, 2], [5, -2 ** 31])
