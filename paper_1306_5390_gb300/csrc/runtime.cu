@@ -849,10 +849,12 @@ int run_hybrid(hgrms_ctx* h, const BatchImg* im, int n, int alpha, int beta, int
     for (int i = 0; i < n; ++i) all_dev = all_dev && im[i].dev;
     if (h->opt_graph && !ms && !h->coop_stream && all_dev) {
         // Replay the graph of an identical earlier call, or record one.
-        std::vector<uint8_t> key(sizeof(a) + 16 * sizeof(long long));
+        // (the tile kernel too: the same layout sizes can go with another of them)
+        std::vector<uint8_t> key(sizeof(a) + 18 * sizeof(long long));
         memcpy(key.data(), &a, sizeof(a));
-        const long long extra[16] = {beta, T, fused_launches, list_loop, launches, write_back, max_k, n,
-                                     (long long)(uintptr_t)im[0].ptr, im[0].rows, im[0].cols, 0,
+        const long long extra[18] = {beta, T, fused_launches, list_loop, launches, write_back, max_k, n,
+                                     (long long)(uintptr_t)im[0].ptr, im[0].rows, im[0].cols,
+                                     (long long)(uintptr_t)fe, max_rows, max_cols,
                                      timed, bm_total, (long long)(uintptr_t)h->host_ctrl,
                                      (long long)(uintptr_t)h->host_img_k};
         memcpy(key.data() + sizeof(a), extra, sizeof(extra));

@@ -150,3 +150,35 @@ def test_predicted_schedule_as_graph(oracle_mod, torch_cuda):
                 assert st["k_pred"] >= 0, st
                 assert st["graph"] == (2 if rep == 0 else 1), st
                 assert np.array_equal(t.cpu().numpy(), ref)
+
+
+def test_batches_that_differ_in_the_tile_kernel_alone(oracle_mod, torch_cuda):
+    """Two batches with the same first image, pixels, bitmap words and tile
+    count, one of 32-row and one of 64-row tiles (a fixed in-tile switch point
+    and no tensor maps leave nothing else to tell them apart): the second one
+    records a graph of its own."""
+    from paper_1306_5390_gb300 import hgrms
+    torch = torch_cuda
+    n = 60
+    low = [(54, 240)] * n
+    high = [(54, 240)] + [(54, 241)] * 30 + [(54, 239)] * 28 + [(54, 238)]
+    assert sum(r * c for r, c in low) == sum(r * c for r, c in high)
+    base = noisy(54, 241, 0.3, 8600)
+    refs = {c: oracle_mod.denoise(np.ascontiguousarray(base[:, :c]), 10, 1, 32) for c in (238, 239, 240, 241)}
+    buf = torch.empty(n * 54 * 256, dtype=torch.uint8, device="cuda")
+    with hgrms.Denoiser(0) as d:
+        d.set_option(hgrms.HGRMS_OPT_TILE_EVAL_MAX, 4096)
+        d.set_option(hgrms.HGRMS_OPT_TMA, 0)
+        seen = []
+        for graph, shapes in ((0, high), (0, low), (1, low), (1, high), (1, low), (1, high)):
+            d.set_option(hgrms.HGRMS_OPT_GRAPH, graph)
+            ts = [buf[i * 54 * 256:i * 54 * 256 + r * c].view(r, c) for i, (r, c) in enumerate(shapes)]
+            for t in ts:
+                t.copy_(torch.from_numpy(np.ascontiguousarray(base[:, :t.shape[1]])))
+            ks = d.denoise_batch(ts, 10, 1, 32)
+            st = d.stats()
+            seen.append((st["graph"], st["tile_rows"], st["ctas_per_launch"]))
+            for t, k in zip(ts, ks):
+                ref, k_ref, _ = refs[t.shape[1]]
+                assert k == k_ref and np.array_equal(t.cpu().numpy(), ref), (graph, tuple(t.shape), seen)
+    assert seen == [(0, 50, 180), (0, 18, 180), (2, 18, 180), (2, 50, 180), (1, 18, 180), (1, 50, 180)]
