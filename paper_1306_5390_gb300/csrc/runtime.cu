@@ -518,14 +518,22 @@ int default_eval_max(int beta) {
     return beta == 2 ? 2048 : 4096;
 }
 
-// Canvas, bitmap and list bytes the hybrid schedule needs for one image (a
-// chunk needs the sum, plus a small constant).
-long long hybrid_bytes(const hg::FusedEntry* fe, int rows, int cols) {
-    const long long tiles_x = (cols + fe->TW - 1) / fe->TW, tiles_y = (rows + fe->TH - 1) / fe->TH;
-    const long long pitch = (hg::kPadX + tiles_x * fe->TW + 16 + 127) / 128 * 128;
-    const long long crows = hg::kPadY + tiles_y * fe->TH + 16;
+// Canvas, bitmap, list and tile map bytes the hybrid schedule needs for one
+// image with the tiles that take most of them, as the choice among the tile
+// heights depends on the other images of the chunk (a chunk needs the sum,
+// plus a small constant).
+long long hybrid_bytes(int beta, int T, int rows, int cols) {
     const long long px = (long long)rows * cols;
-    return 3 * pitch * crows + 4 * 4 * (long long)rows * ((cols + 31) / 32 + 1) + 4 * 4 * (px / 4) + 4 * tiles_x * tiles_y;
+    long long tiled = 0;
+    for (int rn : {32, 64, 128}) {
+        const hg::FusedEntry* fe = find_fused(beta, T, rn);
+        if (!fe) continue;
+        const long long tiles_x = (cols + fe->TW - 1) / fe->TW, tiles_y = (rows + fe->TH - 1) / fe->TH;
+        const long long pitch = (hg::kPadX + tiles_x * fe->TW + 16 + 127) / 128 * 128;
+        const long long crows = hg::kPadY + tiles_y * fe->TH + 16;
+        tiled = std::max(tiled, 3 * pitch * crows + 4 * tiles_x * tiles_y);
+    }
+    return tiled + 4 * 4 * (long long)rows * ((cols + 31) / 32 + 1) + 4 * 4 * (px / 4);
 }
 
 // Tensor maps for the fused kernel's TMA tile loads of one call (kernel `fe`,
@@ -1386,8 +1394,7 @@ HG_EXPORT int hgrms_denoise_batch(hgrms_t h, uint8_t* const* imgs, const int* ro
         // chunk ends before the image that would exceed the memory budget,
         // the image count of one launch or the 32-bit change-list packing.
         const int T = h->opt_passes > 0 ? h->opt_passes : default_passes(beta);
-        const hg::FusedEntry* fe = find_fused(beta, T);
-        if (!fe) return HGRMS_EINVAL;
+        if (!find_fused(beta, T)) return HGRMS_EINVAL;
         const long long budget = (long long)(h->opt_batch_mb > 0 ? h->opt_batch_mb : 8192) << 20;
         h->stats = hgrms_stats_t{};
         h->stats.k_pred = -1.0;
@@ -1396,7 +1403,7 @@ HG_EXPORT int hgrms_denoise_batch(hgrms_t h, uint8_t* const* imgs, const int* ro
             int end = start, mr = 1, mc = 1;
             long long bytes = 0;
             while (end < n) {
-                const long long nb = hybrid_bytes(fe, rows[end], cols[end]);
+                const long long nb = hybrid_bytes(beta, T, rows[end], cols[end]);
                 const int mr2 = rows[end] > mr ? rows[end] : mr, mc2 = cols[end] > mc ? cols[end] : mc;
                 const int cnt = end - start + 1;
                 const bool fits = cnt <= hg::kMaxBatchImages && bytes + nb <= budget &&

@@ -55,12 +55,14 @@ struct Request {
 };
 
 // Device bytes one request needs while served: its resident copy (host
-// requests) plus what the batched schedule allocates per pixel (three
-// canvases with padding, four change lists and bitmaps; an upper estimate).
+// requests) plus what the batched schedule allocates for it (three canvases
+// of whole tiles, which end less than 128 rows and 240 columns behind the
+// image, with borders and rows of whole 128 bytes; four change lists and
+// bitmaps; an upper estimate).
 long long request_bytes(int rows, int cols, bool device) {
     const long long px = (long long)rows * cols;
-    const long long padded = (long long)(rows + 96) * (long long)(cols + 288);
-    return (device ? 0 : px) + 3 * padded + 4 * px + px / 2 + 4096;
+    const long long padded = (long long)(rows + 127 + 32) * (long long)(cols + 239 + 32 + 127);
+    return (device ? 0 : px + 255) + 3 * padded + 4 * px + px / 2 + 32ll * rows + 4096;
 }
 
 }  // namespace

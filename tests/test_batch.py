@@ -307,3 +307,32 @@ def test_tall_tiles_of_mid_sized_batches(oracle_mod, den, torch_cuda, n, rows, c
     tall = tiles[128] >= 2 * sms and -(-tiles[128] // sms) * 10 <= tiles[64] // (2 * sms) * 10 + (
         0 if rest == 0 else 6 if rest <= sms else 10) and tiles[128] * 128 < tiles[64] * 64
     assert den.stats()["tile_rows"] == (128 if tall else 64) - 2 * (T - 1) * beta
+
+
+def test_chunks_stay_within_the_memory_budget(oracle_mod, torch_cuda):
+    """2000 images, half of which the batch's 128-row tiles pad by far more than
+    64-row ones would (115 rows: 228 against 150), with a budget for some 1400
+    of them: what the handle allocates stays within the budget (the lists' 64 Ki
+    spare entries, the tables and 2 MiB of rounding for each of the handle's
+    buffers aside)."""
+    from paper_1306_5390_gb300 import hgrms
+    torch = torch_cuda
+    n, cols, mb = 2000, 481, 1000
+    base = synth.noisy_image(115, cols, 0.3, 960)[1]
+    refs = {r: oracle_mod.denoise(np.ascontiguousarray(base[:r]), 10, 1, 16) for r in (114, 115)}
+    sizes = [114 if i % 50 < 26 else 115 for i in range(n)]
+    work = torch.from_numpy(base).cuda().repeat(n, 1, 1)
+    views = [w[:r] for w, r in zip(work, sizes)]
+    with hgrms.Denoiser(0) as d:
+        d.denoise(work[0].clone(), 10, 1, 16)  # code and the handle's fixed buffers
+        d.set_option(hgrms.HGRMS_OPT_BATCH_MB, mb)
+        torch.cuda.synchronize()
+        before = torch.cuda.mem_get_info()[0]
+        ks = d.denoise_batch(views, 10, 1, 16)
+        torch.cuda.synchronize()
+        used = before - torch.cuda.mem_get_info()[0]
+        assert d.stats()["tile_rows"] == 128 - 14 and d.stats()["launches"] == 4
+    out = {r: torch.from_numpy(refs[r][0]).cuda() for r in refs}
+    assert ks == [refs[r][1] for r in sizes]
+    assert all(bool((v == out[r]).all()) for v, r in zip(views, sizes))
+    assert used <= (mb + 24) << 20, used / 2**20
