@@ -327,11 +327,8 @@ struct Plan {
     int tiles_x, tiles_y;
     long long pitch;
     long long crows;
-    int launches;       // all launches
-    int fused_launches; // of which fused
+    int launches;
     int map_words;
-    size_t list_cap;
-    int bm_words;
 };
 
 // Launch plan of the unfused and fused-only schedules (the hybrid schedule
@@ -341,8 +338,6 @@ int make_plan(hgrms_ctx* h, int rows, int cols, int beta, int max_k, Plan* p) {
     if (p->schedule == kHybrid) return HGRMS_EINVAL;
     p->fused = p->schedule != kPlain;
     p->fe = nullptr;
-    p->list_cap = 0;
-    p->bm_words = 0;
     if (p->fused) {
         p->T = h->opt_passes > 0 ? h->opt_passes : default_passes(beta);
         p->fe = find_fused(beta, p->T);
@@ -352,7 +347,7 @@ int make_plan(hgrms_ctx* h, int rows, int cols, int beta, int max_k, Plan* p) {
         const long long need_w = hg::kPadX + (long long)p->tiles_x * p->fe->TW + 16;
         p->pitch = (need_w + 127) / 128 * 128;
         p->crows = hg::kPadY + (long long)p->tiles_y * p->fe->TH + 16;
-        p->fused_launches = p->launches = (max_k + p->T - 1) / p->T;
+        p->launches = (max_k + p->T - 1) / p->T;
         p->map_words = (p->tiles_x * p->fe->TW + 31) / 32 + 2;
     } else {
         p->T = 1;
@@ -361,7 +356,6 @@ int make_plan(hgrms_ctx* h, int rows, int cols, int beta, int max_k, Plan* p) {
         p->pitch = (need_w + 127) / 128 * 128;
         p->crows = hg::kPadY + (long long)rows + 16;
         p->launches = max_k;
-        p->fused_launches = 0;
         p->map_words = 0;
     }
     return HGRMS_OK;
@@ -1060,11 +1054,6 @@ int denoise_one(hgrms_ctx* h, uint8_t* img, int rows, int cols, int alpha, int b
         rc = ensure_maps(h, 3 * map_bytes);
         if (rc < 0) return rc;
     }
-    const size_t bm_size = (size_t)rows * (size_t)p.bm_words;
-    if (p.list_cap > 0) {
-        rc = ensure_lists(h, p.list_cap, bm_size);
-        if (rc < 0) return rc;
-    }
     cudaStream_t s = h->stream;
     uint8_t* ca = h->canvas[0];
     if (dev) {
@@ -1076,12 +1065,8 @@ int denoise_one(hgrms_ctx* h, uint8_t* img, int rows, int cols, int alpha, int b
     HG_TRY(h, hg::launch_call_init(h->ctrl, (unsigned)max_k, nullptr, 0, nullptr, nullptr, 0, h->sms, s));
     // Map 0 is written by the first launch; the launches clear the others.
     if (p.map_words > 0) HG_TRY(h, cudaMemsetAsync(h->chg_maps, 0, map_bytes, s));
-    // The change bitmaps start empty; each list pass clears one for a later pass.
-    if (p.list_cap > 0) {
-        HG_TRY(h, cudaMemsetAsync(h->bitmaps, 0, 4 * bm_size * sizeof(uint32_t), s));
-        HG_TRY(h, cudaMemsetAsync(h->bar, 0, sizeof(hg::GridBar), s));
-    }
     hg::PassArgs a;
+    memset(&a, 0, sizeof(a));
     for (int i = 0; i < 3; ++i) a.canvas[i] = h->canvas[i];
     a.pitch = p.pitch;
     a.rows = rows;
@@ -1091,28 +1076,10 @@ int denoise_one(hgrms_ctx* h, uint8_t* img, int rows, int cols, int alpha, int b
     a.ctrl = h->ctrl;
     a.chg_maps = p.map_words > 0 ? h->chg_maps : nullptr;
     a.map_words = p.map_words;
-    for (int i = 0; i < 4; ++i) {
-        a.lists[i] = p.list_cap > 0 ? h->lists + i * p.list_cap : nullptr;
-        a.bitmaps[i] = p.list_cap > 0 ? h->bitmaps + i * bm_size : nullptr;
-    }
-    a.list_cap = (unsigned)p.list_cap;
-    a.bm_words = p.bm_words;
-    a.bar = h->bar;
-    a.write_prev = 0;
-    a.imgs = nullptr;
     a.nimg = 1;
     a.xb = a.yb = 16;
-    a.tile_img = nullptr;
-    a.bm_total = 0;
-    a.img_k = nullptr;
     a.ntiles = p.tiles_x * p.tiles_y;
-    a.hybrid = 0;
-    a.relaunch_evals = 0;
     a.tile_eval_max = h->opt_tile_eval_max;
-    a.user0 = nullptr;
-    a.list_ctas = 0;
-    a.bar_extra = h->opt_wait_test > 0 ? 1u : 0u;
-    a.bar_spins = (unsigned)h->opt_wait_test;
     // Per-launch timing is limited to calls of at most kMaxTimedLaunches launches.
     constexpr int kMaxTimedLaunches = 4096;
     const bool timed = h->opt_timing && p.launches <= kMaxTimedLaunches;
@@ -1122,10 +1089,8 @@ int denoise_one(hgrms_ctx* h, uint8_t* img, int rows, int cols, int alpha, int b
     }
     for (int i = 0; i < p.launches; ++i) {
         if (timed) HG_TRY(h, cudaEventRecord(h->events[2 * i], s));
-        if (i < p.fused_launches)
+        if (p.fused)
             HG_TRY(h, p.fe->launch(a, p.tiles_x * p.tiles_y, s));
-        else if (p.fused)
-            HG_TRY(h, chain_coop(h, s, [&] { return hg::launch_list(beta, a, h->sms, s); }));
         else
             HG_TRY(h, hg::launch_plain(beta, a, s));
         if (timed) HG_TRY(h, cudaEventRecord(h->events[2 * i + 1], s));
