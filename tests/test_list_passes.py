@@ -251,6 +251,45 @@ def test_short_lists_that_outlive_a_round_of_one_cta(oracle_mod, den, torch_cuda
             assert np.array_equal(t.cpu().numpy(), ref[0])
 
 
+# Images whose lists cross the line to one CTA's passes and back: (beta, alpha,
+# rows, columns, density, seed, how often they come back).
+CROSSING = [(1, 2, 108, 57, 0.105, 229, 1), (3, 1, 114, 113, 0.304, 51, 1), (5, 0, 88, 33, 0.516, 97, 2),
+            (5, 1, 109, 74, 0.640, 223, 2)]
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("beta,alpha,rows,cols,density,seed,back", CROSSING)
+def test_lists_go_back_from_one_cta_to_the_grid(oracle_mod, den, torch_cuda, beta, alpha, rows, cols, density, seed, back):
+    """Lists that get longer than one CTA takes after passes that it ran, once
+    and twice: the image alone, in batches beside images that do not change and
+    beside a copy of itself, calls that end around the crossings."""
+    from paper_1306_5390_gb300 import hgrms
+    img = synth.noisy_image(rows, cols, density, seed)[1]
+    still = np.full((90, 140), 100, np.uint8)
+    first, _ = oracle_mod.one_pass(img, alpha, beta)
+    line = 112 if beta == 1 else 2048 // (2 * beta + 1) ** 2
+    sizes = []
+    list_passes(oracle_mod, first, img, 1, alpha, beta, 60, 6, sizes=sizes)
+    short = [n <= line for n in sizes]
+    at = [i for i in range(len(short) - 1) if short[i] and not short[i + 1]]
+    assert len(at) >= back
+    den.set_option(hgrms.HGRMS_OPT_PASSES, 1)
+    try:
+        for max_k in sorted({60, 1 + at[0], 2 + at[0], 3 + at[0], 4 + at[-1]}):
+            ref, k_ref, c_ref = oracle_mod.denoise(img, alpha, beta, max_k)
+            t = torch_cuda.from_numpy(img.copy()).cuda()
+            assert den.denoise(t, alpha, beta, max_k) == k_ref and den.converged() == c_ref
+            assert np.array_equal(t.cpu().numpy(), ref)
+            for batch in ([still, img, still], [still] * 40 + [img], [img, img]):
+                ts = [torch_cuda.from_numpy(im.copy()).cuda() for im in batch]
+                ks = den.denoise_batch(ts, alpha, beta, max_k)
+                for im, t, k in zip(batch, ts, ks):
+                    assert k == (0 if im is still else k_ref)
+                    assert np.array_equal(t.cpu().numpy(), still if im is still else ref)
+    finally:
+        den.set_option(hgrms.HGRMS_OPT_PASSES, 0)
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("cols", [225, 239, 240, 241, 255, 257, 480])
 @pytest.mark.parametrize("beta", [1, 2, 3])
