@@ -92,11 +92,14 @@ def test_features_match_definition(torch_cuda):
 
 
 @pytest.mark.parametrize("rows,cols", [(1, 70), (63, 64), (129, 65), (70, 127), (64, 128), (130, 129), (66, 1023),
-                                              (65, 1025), (300, 259), (16500, 64), (20000, 3), (40, 4100)])
+                                              (65, 1025), (300, 259), (16500, 64), (20000, 3), (40, 4100), (70, 511),
+                                              (71, 512), (72, 513), (16500, 1030), (33000, 520), (65536, 64)])
 def test_features_at_the_ends_of_their_ranges(torch_cuda, rows, cols, offset=1):
-    """Widths around a warp's columns and a lane's four, rows past the 256 a
-    16-bit sum holds, constant images (one histogram bin, full counters), odd
-    addresses.  Sums are whole numbers; the division rounds once (1e-6)."""
+    """Widths around a lane's 16 columns and a warp's 512, bands of more rows
+    than the 255 a 16-bit sum holds for a warp that takes every row of its
+    columns, every second and every fourth (16500 x 1030, 33000 x 520, 65536 x
+    64), constant images (one histogram bin, full counters), odd addresses.
+    Sums are whole numbers; the division rounds once (1e-6)."""
     torch = torch_cuda
     from paper_1306_5390_gb300 import hgrms
     rng = np.random.Generator(np.random.PCG64(rows + cols))
