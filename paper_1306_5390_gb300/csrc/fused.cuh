@@ -963,14 +963,14 @@ fused_kernel(PassArgs a) {
 
     // Launch-wide clearing, shared by all CTAs: the map the next launch
     // writes, or the change set the next launch writes (its bitmap, by
-    // walking its list, or all of it after an overflow).
+    // walking its list, or all of it after an overflow or when the list is longer).
     {
         const size_t gt = (size_t)gridDim.x * G::kThreads, gi = (size_t)blockIdx.x * G::kThreads + tid;
         for (size_t i = gi; i < map_size; i += gt) map_clr[i] = 0u;  // map_size is 0 without maps
         if (a.hybrid) {
             uint32_t* bm = a.bitmaps[set_clr];
             const unsigned nclr = s_nclr;
-            if (nclr <= a.list_cap) {
+            if (nclr <= a.list_cap && nclr <= a.bm_total) {
                 const uint32_t* lst = a.lists[set_clr];
                 for (size_t i = gi; i < nclr; i += gt) {
                     unsigned im;

@@ -614,11 +614,12 @@ __global__ void __launch_bounds__(kListThreads, 2) list_loop_kernel(PassArgs a) 
             if (i0 < (long long)n * per) pk_first = __ldcg(prev + (unsigned)(i0 / per));
         }
         // Clear bitmap sc (written by pass t - 2, read by pass t - 1) for pass
-        // t + 2: walk its list, or clear it all if the list overflowed.
+        // t + 2: walk its list, or clear it all if the list overflowed or is
+        // longer than the bitmap.
         {
             const uint32_t* clr = a.lists[sc];
             uint32_t* bm_clr = a.bitmaps[sc];
-            if (nclr <= a.list_cap) {
+            if (nclr <= a.list_cap && nclr <= a.bm_total) {
                 for (long long i = gtid; i < nclr; i += gthreads) {
                     unsigned img;
                     int y, x;
