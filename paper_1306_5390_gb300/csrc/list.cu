@@ -24,11 +24,11 @@
 // D_(t+1) and can make either; a pass that reads D_t can make only D_(t+1).  D_t
 // holds C_(t-1)'s settled pixels too, so while the changes still die out C is the
 // shorter list.  make_c draws the line: C again while the last list was
-// shorter than 3/4 (short lists 3/5) of the one before it, and in the first
-// pass, which knows no ratio (beta 5, 1000 x 1500, 2 % impulses: 1.5 M
-// evaluations against 2.8 M with D from the first pass on; 8192 x 8192, beta 2
-// 0.94 ms a call against 1.00; beta 1, where eight passes have run by then,
-// 0.917 against 0.919).  Lists of more than 1/32 of the pixels are no oscillations
+// shorter than 3/4 (short lists 3/5) of the one before it (beta 5, 1000 x
+// 1500, 2 % impulses: 1.5 M evaluations against 2.8 M with D from the first
+// pass on); the first pass, which knows no ratio, makes D when the fused
+// launches ran kDirectD passes, by then the changes left are mostly
+// oscillations.  Lists of more than 1/32 of the pixels are no oscillations
 // yet: they make C while they shrink at all (textured 4096 x 4096, 70 %
 // impulses, beta 3: alpha 1 4.17 ms a call against 5.16 when D began at once, alpha
 // 2 1.75 against 2.15; 8192 x 8192, alpha 2, beta 1: 6.5 against 7.4), and with
@@ -285,6 +285,7 @@ __device__ __forceinline__ void add_image(int* img_n, int d, unsigned img, int l
 // left to CTA 0 alone, with the lists and the claims in shared memory: 1.25 us
 // a pass for 30 pixels of beta 2, 2.4 us for 44, 5.4 us for 205 of beta 1 (four
 // rounds of the CTA's threads, where the grid is faster again).
+constexpr unsigned kDirectD = 6;
 constexpr int kDirectB = 2;
 constexpr int kDescCache = 128;
 constexpr int kSoloEvals = 2048;
@@ -306,12 +307,12 @@ struct LoopState {
     unsigned n_before;  // entries of the list that the last pass read (0: no pass yet)
     bool c_list;        // the next pass reads C_t (else D_t)
     // Whether the next pass, from a list of n entries, makes C (see the header;
-    // dense: 1/32 of the pixels).
-    __device__ __forceinline__ bool make_c(unsigned n, unsigned dense, int alpha) const {
-        if (!c_list || n_before == 0u) return c_list;
+    // k0: passes before this launch, dense: 1/32 of the pixels).
+    __device__ __forceinline__ bool make_c(unsigned n, unsigned k0, unsigned dense, int alpha) const {
+        if (!c_list) return false;
         const unsigned long long now = n, before = n_before;
-        if (n > dense && (now * 16u < before * 15u || (alpha == 0 && n / 4u > dense))) return true;
-        return n > kShortList ? now * 4u < before * 3u : now * 5u < before * 3u;
+        if (n > dense && (n_before == 0u || now * 16u < before * 15u || (alpha == 0 && n / 4u > dense))) return true;
+        return n_before == 0u ? k0 < kDirectD : (n > kShortList ? now * 4u < before * 3u : now * 5u < before * 3u);
     }
 };
 
@@ -327,7 +328,7 @@ struct LoopState {
 // counters; dn accumulates this thread's share of the change of N.
 template <int B, bool kBatch>
 __device__ __forceinline__ void solo_passes(const PassArgs& a, const ImgDesc& one, const int base, const int xb,
-                                            const int yb, const unsigned max_k, LoopState& st, uint32_t* lists,
+                                            const int yb, const unsigned max_k, const unsigned k0, LoopState& st, uint32_t* lists,
                                             uint32_t* hash, unsigned* s_n, unsigned& evals, int& dn) {
     constexpr int W = 2 * B + 1, P = W * W, NW = (W + 3) / 4;
     const int tid = threadIdx.x;
@@ -359,7 +360,7 @@ __device__ __forceinline__ void solo_passes(const PassArgs& a, const ImgDesc& on
         const uint8_t* in_arena = a.canvas[st.cur];
         uint8_t* out_arena = a.canvas[st.aux];
         const int ntask = (int)n * P;
-        const bool make_c = st.make_c(n, a.list_dense, a.alpha);
+        const bool make_c = st.make_c(n, k0, a.list_dense, a.alpha);
         for (int i = tid; i < ntask; i += kListThreads) {
             const int e = i / P, o = i - e * P;
             unsigned img;
@@ -536,7 +537,7 @@ __global__ void __launch_bounds__(kListThreads, 2) list_loop_kernel(PassArgs a) 
         if (st.n_cur <= kSoloPixels<B> && st.n_cur <= a.list_cap && st.n_last <= kSoloClear &&
             st.n_last <= a.list_cap) {
             if (blockIdx.x == 0) {
-                solo_passes<B, kBatch>(a, one, base, xb, yb, max_k, st, stage_all, s_queue, s_solo_n, evals, dn);
+                solo_passes<B, kBatch>(a, one, base, xb, yb, max_k, k0, st, stage_all, s_queue, s_solo_n, evals, dn);
                 dn = __reduce_add_sync(0xffffffffu, dn);
                 if (lane == 0 && dn) atomicAdd(&s_dn, dn);
                 __syncthreads();
@@ -589,7 +590,7 @@ __global__ void __launch_bounds__(kListThreads, 2) list_loop_kernel(PassArgs a) 
         uint32_t* next = a.lists[so];
         uint32_t* bm_next = a.bitmaps[so];
         unsigned* nnext = &ctrl->list_n[so];
-        const bool make_c = st.make_c(st.n_cur, a.list_dense, a.alpha);
+        const bool make_c = st.make_c(st.n_cur, k0, a.list_dense, a.alpha);
         // N is needed from the first D_t on: the pass that makes it counts the
         // pixels it changes, the later ones the differences.
         const int add = make_c ? 0 : 1, sub = st.c_list ? 0 : 1;

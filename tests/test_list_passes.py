@@ -31,17 +31,17 @@ def dilate(m, b):
 def makes_c(n, before, alpha, k0, c_first_below, dense, short):
     """Whether a pass that reads a list C of n pixels makes C again (before: the
     length of the list before it, 0 for the first pass)."""
+    if n > dense and (before == 0 or n * 16 < before * 15 or (alpha == 0 and n // 4 > dense)):
+        return True
     if before == 0:
         return k0 < c_first_below
-    if n > dense and (n * 16 < before * 15 or (alpha == 0 and n // 4 > dense)):
-        return True
     return n * 4 < before * 3 if n > short else n * 5 < before * 3
 
 
 def list_passes(oracle_mod, cur, aux, k, alpha, beta, max_k, c_first_below, sizes=None, dense=1 << 30, short=4096):
     """The loop from I_k = cur and I_(k-1) = aux on: (image, k, converged).
-    c_first_below: the first pass makes C when k is below it (the kernel's
-    always does); longer lists than dense and short follow other lines.  sizes, when given, receives the length
+    c_first_below: the first pass makes C when k is below it; longer lists than
+    dense and short follow other lines.  sizes, when given, receives the length
     of the list that each pass reads."""
     rows, cols = cur.shape
     inner = np.zeros((rows, cols), dtype=bool)
@@ -269,7 +269,7 @@ def test_lists_go_back_from_one_cta_to_the_grid(oracle_mod, den, torch_cuda, bet
     first, _ = oracle_mod.one_pass(img, alpha, beta)
     line = 112 if beta == 1 else 2048 // (2 * beta + 1) ** 2
     sizes = []
-    list_passes(oracle_mod, first, img, 1, alpha, beta, 60, 99, sizes=sizes)
+    list_passes(oracle_mod, first, img, 1, alpha, beta, 60, 6, sizes=sizes)
     short = [n <= line for n in sizes]
     at = [i for i in range(len(short) - 1) if short[i] and not short[i + 1]]
     assert len(at) >= back
