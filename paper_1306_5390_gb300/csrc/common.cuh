@@ -258,7 +258,10 @@ __device__ __forceinline__ int warp_excl_scan(const int lane, const int n, int* 
 // Programmatic dependent launches.  A launch made with launch_dependent may
 // become resident before the launch ahead of it in its stream has ended: it
 // must reach wait_for_previous before it touches memory (the wait lasts until
-// that launch has completed and its writes are visible; no-op otherwise).
+// that launch has completed and its writes are visible; no-op otherwise).  An
+// event wait in between, as before a server slot's last launch, whose list-pass
+// launch runs on another stream, orders it behind the event as any launch: only
+// the launch ahead in its own stream may still be running.
 // let_next_start, in the launch ahead, allows that from there on.  Used for a
 // call's fused launches (behind the init launch) and its last one: a call loses
 // 3 to 5 us of launch latency (256 x 256 52.5 -> 49.1 us, 3839 x 2161 136 -> 131).

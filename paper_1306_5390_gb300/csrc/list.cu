@@ -284,7 +284,15 @@ __device__ __forceinline__ void add_image(int* img_n, int d, unsigned img, int l
 // which the barrier is about 2 us.  Lists of at most kSoloPixels pixels are
 // left to CTA 0 alone, with the lists and the claims in shared memory: 1.25 us
 // a pass for 30 pixels of beta 2, 2.4 us for 44, 5.4 us for 205 of beta 1 (four
-// rounds of the CTA's threads, where the grid is faster again).
+// rounds of the CTA's threads, where the grid is faster again).  kSoloPixels: twice as many
+// for beta 1 cost 8192 x 8192 20 us more a call, half as many 64 photographs 8 us and
+// 1000 x 1000 3 us; for beta 2 and 3 (four rounds) half as many measured the
+// same on 700 x 900 to 8192 x 8192.  kDescCache: 64 and 256 entries measured like
+// 128 on batches of 64 to 512 images (128 take 6 KB).  kDirectD lies between
+// beta 2's four fused passes (8192 x 8192 0.94 ms a call; 1.00 with D in the first
+// list pass) and beta 1's eight, where D gains on one image and photographs
+// (0.914 against 0.918 ms, 0.599 against 0.604) and loses on uneven ones (128 of
+// them 3.00 ms against 2.95).
 constexpr unsigned kDirectD = 6;
 constexpr int kDirectB = 2;
 constexpr int kDescCache = 128;
@@ -316,7 +324,7 @@ struct LoopState {
     }
 };
 
-// Passes run by CTA 0 alone, from a list of st.n_cur <= kSoloEvals / P
+// Passes run by CTA 0 alone, from a list of st.n_cur <= kSoloPixels<B>
 // pixels, until a list comes out empty, k reaches max_k, a list is longer
 // than that or kSoloPasses passes have run (the other CTAs wait meanwhile, and
 // their wait is bounded).  One thread takes one (listed pixel, window
@@ -331,6 +339,7 @@ __device__ __forceinline__ void solo_passes(const PassArgs& a, const ImgDesc& on
                                             const int yb, const unsigned max_k, const unsigned k0, LoopState& st, uint32_t* lists,
                                             uint32_t* hash, unsigned* s_n, unsigned& evals, int& dn) {
     constexpr int W = 2 * B + 1, P = W * W, NW = (W + 3) / 4;
+    static_assert(kSoloPixels<B> * P <= kSoloEvals, "the next list and the claim table hold every window position");
     const int tid = threadIdx.x;
     uint32_t* list = lists;
     uint32_t* next = lists + kSoloEvals;

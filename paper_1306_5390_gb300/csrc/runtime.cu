@@ -176,11 +176,13 @@ namespace {
 // Hybrid schedule: fused launches after the first (each runs only when the
 // previous one left many changed pixels; a launch that does not run still
 // costs 4 to 6 us).  With alpha >= 2 the list passes take over after the first
-// launch whatever it left, because their lists shrink by about half per pass
-// (list.cu): 128 images of 128..2048 pixels a side, 5..70 % impulses, 3.39 ms
+// launch whatever it left, because their lists shrink (list.cu), with alpha 10 by
+// about half per pass: 128 images of 128..2048 pixels a side, 5..70 % impulses, 3.39 ms
 // a call without relaunches against 3.75 ms with one and 5.14 ms with three;
 // 8192 x 8192 at 70 % 2.18 against 2.55 and 3.77 ms; 2048 x 2048 at 50 % 0.349
-// against 0.366 and 0.396 ms.  With alpha 0 every interior pixel is replaced
+// against 0.366 and 0.396 ms.  Near the line, textured 8192 x 8192: alpha 2 7.81
+// ms at 30 % impulses and 6.29 at 70 % (8.22 and 6.19 with three), alpha 3 3.7
+// and 5.2 (4.9 and 5.9).  With alpha 0 every interior pixel is replaced
 // in every pass and no list shrinks, and with alpha 1 the lists of a noise
 // image shrink slowly (18 % of the pixels after 8 passes): there, for beta 1
 // (T = 8, the cheapest fused pass) and large calls, up to 3 of them run when a
