@@ -382,8 +382,8 @@ typedef struct hgrms_stats {
                                (every image pixel per dense pass, else the pixels within
                                beta of a change of the previous pass) */
     long long evals_list;   /* the same for list-pass launches: the pixels whose window
-                               differs from the one two passes back (or, in their first
-                               passes, one pass back) */
+                               differs from the one two passes back (while the changes die
+                               out, one pass back); every pixel where most windows do */
     int    tile_eval_max;   /* in-tile list/dense switch point used (HGRMS_OPT_TILE_EVAL_MAX) */
     int    autotuned;       /* 1 if the tuning came from the autotuner (HGRMS_OPT_AUTOTUNE) */
     double tune_ms;         /* device time the autotuner's trials took in this call (0 when the
