@@ -28,12 +28,15 @@
 // 1500, 2 % impulses: 1.5 M evaluations against 2.8 M with D from the first
 // pass on); the first pass, which knows no ratio, makes D when the fused
 // launches ran kDirectD passes, by then the changes left are mostly
-// oscillations.  Lists of more than 1/32 of the pixels are no oscillations
-// yet: they make C while they shrink at all (textured 4096 x 4096, 70 %
-// impulses, beta 3: alpha 1 4.17 ms a call against 5.16 when D began at once, alpha
-// 2 1.75 against 2.15; 8192 x 8192, alpha 2, beta 1: 6.5 against 7.4), and with
-// alpha 0, which replaces every interior pixel in every pass, however they
-// shrink (1024 x 1024, beta 1: 0.64 ms against 0.75).
+// oscillations.  (3/4 for lists of some thousand pixels too: 1024 x 1024, 70 %
+// impulses, beta 2, 75 us against 70; 3/5 for all: textured 4096 x 4096, alpha 1,
+// beta 3, 3.31 ms against 3.13.)  Lists of more than 1/32 of the pixels are no
+// oscillations yet: they make C while they shrink at all (textured 4096 x
+// 4096, 70 % impulses, beta 3: alpha 1 4.17 ms a call against 5.16 when D began at
+// once, alpha 2 1.75 against 2.15; 8192 x 8192, alpha 2, beta 1: 6.5 against 7.4;
+// with the line at 1/16 alpha 2, beta 3 is 23 % slower, with 1/64 8192 x 8192, alpha
+// 10, 70 % 9 %), and with alpha 0, which replaces every interior pixel in every
+// pass, however they shrink (1024 x 1024, beta 1: 0.64 ms against 0.75).
 //
 // k and the converged flag need to know whether a pass changed the image,
 // N_t = #{q : I_t(q) != I_(t-1)(q)} > 0.  For a pixel that is not evaluated
@@ -610,9 +613,12 @@ __global__ void __launch_bounds__(kListThreads, 2) list_loop_kernel(PassArgs a) 
             ctrl->list_n[(st.t + base + 2) & 3] = 0u;
         }
         const unsigned n = st.n_cur, nclr = st.n_last;
-        // The windows of an eighth of the pixels hold nearly all of them: for
-        // beta >= 2 a pass over every pixel costs less than one by such a list.
-        const bool whole = n > a.list_cap || (B > 1 && n / 4u > a.list_dense);
+        // The windows of a sixteenth of the pixels hold most of them: for beta
+        // >= 2 a pass over every pixel costs less than one by such a list.  Lines at
+        // 1/8, 1/16 and 1/32 of the pixels: textured 4096 x 4096, alpha 1, beta 3,
+        // 30 % impulses 3.03, 2.39 and 2.41 ms a call, alpha 2, beta 2, 70 % 1.38, 1.18
+        // and 1.24; for beta 1 1/8 measured like the overflow alone.
+        const bool whole = n > a.list_cap || (B > 1 && n / 2u > a.list_dense);
         // A short list: one thread per (listed pixel, window position).
         const bool direct = B <= kDirectB && (long long)n * P <= gthreads && !whole;
         // The list entry of this thread's first task, loaded before the bitmap clearing below so that the two

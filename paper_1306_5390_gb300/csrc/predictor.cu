@@ -566,7 +566,8 @@ __global__ void __launch_bounds__(kHeadThreads) head_kernel(const __nv_bfloat16*
 // descriptor).  Six accumulators of 16 columns, and one with a matrix of
 // ones as A for db, stay in tensor memory over all tasks of a CTA, one CTA per
 // SM (so an FP32 sum runs over the bands of several images, 1024 positions each,
-// before an atomic adds it to the others'; it ran over one image); the next task's planes load while this one's MMAs run.  One warp
+// before an atomic adds it to the others'; it ran over one image); the next
+// task's planes load while this one's MMAs run.  One warp
 // issues everything.  Bound by the operand reads from shared memory (2 KB per
 // MMA, 7 x 66 MMAs a task, 35 cycles each).  256 images: 58 us; transposing both
 // operands value by value, one 64-position chunk after another, took 190 us.
