@@ -606,7 +606,6 @@ __global__ void __launch_bounds__(kListThreads, 2) list_loop_kernel(PassArgs a) 
         // N is needed from the first D_t on: the pass that makes it counts the
         // pixels it changes, the later ones the differences.
         const int add = make_c ? 0 : 1, sub = st.c_list ? 0 : 1;
-        const bool blind = make_c && st.c_list;
         if (tid == 0 && blockIdx.x == 0) {
             // Set (t + base + 2) % 4 is next written by pass t + 1; its list
             // was last read (to clear its bitmap) in pass t - 1.
@@ -915,12 +914,11 @@ __global__ void __launch_bounds__(kListThreads, 2) list_loop_kernel(PassArgs a) 
                         const int y = (int)(i / d.cols), x = (int)(i - (long long)y * d.cols);
                         const long long off = (long long)y * d.pitch + x;
                         ++evals;
-                        // From C to C what the output holds does not matter: it is written over unread.
-                        const int ip = in[off], was = blind ? ip : __ldcg(out + off);
+                        const int ip = in[off], was = __ldcg(out + off);
                         int nv = ip;
                         if (y >= B && y < d.rows - B && x >= B && x < d.cols - B)
                             nv = eval_pixel<B>(in + off, d.pitch, a.alpha);
-                        if (blind || nv != was) out[off] = (uint8_t)nv;
+                        if (nv != was) out[off] = (uint8_t)nv;
                         if (nv != (make_c ? ip : was)) {
                             ch = true;
                             v = pack_entry((unsigned)im, y, x, xb, yb);
