@@ -31,12 +31,12 @@
 // oscillations.  (3/4 for lists of some thousand pixels too: 1024 x 1024, 70 %
 // impulses, beta 2, 75 us against 70; 3/5 for all: textured 4096 x 4096, alpha 1,
 // beta 3, 3.31 ms against 3.13.)  Lists of more than 1/32 of the pixels are no
-// oscillations yet: they make C while they shrink at all (textured 4096 x
-// 4096, 70 % impulses, beta 3: alpha 1 4.17 ms a call against 5.16 when D began at
-// once, alpha 2 1.75 against 2.15; 8192 x 8192, alpha 2, beta 1: 6.5 against 7.4;
-// with the line at 1/16 alpha 2, beta 3 is 23 % slower, with 1/64 8192 x 8192, alpha
-// 10, 70 % 9 %), and with alpha 0, which replaces every interior pixel in every
-// pass, however they shrink (1024 x 1024, beta 1: 0.64 ms against 0.75).
+// oscillations yet: they make C while they shrink at all (70 % impulses,
+// textured 8192 x 8192, alpha 2, beta 1: 6.28 ms a call against 7.40 when D began at
+// once; 4096 x 4096, alpha 2, beta 3: 1.69 against 2.15, 23 % slower with the line
+// at 1/16; with 1/64 8192 x 8192, alpha 10 is 9 % slower), and with alpha 0, which
+// replaces every interior pixel in every pass, however they shrink (1024 x
+// 1024, beta 1: 0.65 ms against 0.75).
 //
 // k and the converged flag need to know whether a pass changed the image,
 // N_t = #{q : I_t(q) != I_(t-1)(q)} > 0.  For a pixel that is not evaluated
